@@ -416,8 +416,8 @@ tt_fsi_status tt_fsi_masked_game(const tt_fsi_mlp *model, const double *x_dev,
  * estimated with n_background rows (100 in the paper's experiments).
  * background_dev [n_background, d] float64 row-major; layout, types and
  * stream as tt_fsi_masked_game (which is this call with the baseline as the
- * single background row).  One launch per background row; the rows are
- * added in ascending order, so results are deterministic.
+ * single background row).  The rows are added in ascending order, so results
+ * are deterministic.
  */
 tt_fsi_status tt_fsi_masked_game_interventional(const tt_fsi_mlp *model, const double *x_dev,
                                                 const double *background_dev, int n_background, int64_t B,

@@ -14,10 +14,14 @@
 // interventional value function of Section 4.1 (the mean of f over
 // background rows standing in for the absent features) runs as one launch
 // per background row, each adding f / K to v in ascending row order.
+// This kernel serves what the split-digit path (masked_game_split.cu) does
+// not take: hidden widths above 128, fewer than 7 features, and narrow models
+// in float32.
 #include <cuda_runtime.h>
 
 #include <cstdint>
 
+#include "masked_game_split.h"
 #include "tt_fsi.h"
 
 namespace ttfsi_mg {
@@ -126,45 +130,22 @@ __global__ void __launch_bounds__(THREADS) masked_game_kernel(Args a) {
 }  // namespace ttfsi_mg
 
 namespace ttfsi_mg {
-tt_fsi_status masked_game_launch(const tt_fsi_mlp *model, const double *x_dev, const double *baseline_dev, int64_t B,
-                                 void *v_dev, int out_f32, double scale, int accumulate, struct CUstream_st *stream);
-}  // namespace ttfsi_mg
 
-extern "C" tt_fsi_status tt_fsi_masked_game(const tt_fsi_mlp *model, const double *x_dev,
-                                           const double *baseline_dev, int64_t B, void *v_dev,
-                                           int out_f32, struct CUstream_st *stream) {
-    return ttfsi_mg::masked_game_launch(model, x_dev, baseline_dev, B, v_dev, out_f32, 1.0, 0, stream);
-}
-
-extern "C" tt_fsi_status tt_fsi_masked_game_interventional(const tt_fsi_mlp *model, const double *x_dev,
-                                                          const double *background_dev, int n_background, int64_t B,
-                                                          void *v_dev, int out_f32, struct CUstream_st *stream) {
-    if (!model || n_background < 1 || !background_dev) return TT_FSI_ERR_INVALID_ARG;
-    const double scale = 1.0 / (double)n_background;
-    for (int k = 0; k < n_background; ++k) {
-        const tt_fsi_status s = ttfsi_mg::masked_game_launch(model, x_dev, background_dev + (size_t)k * model->d, B,
-                                                             v_dev, out_f32, scale, k > 0, stream);
-        if (s != TT_FSI_OK) return s;
-    }
-    return TT_FSI_OK;
-}
-
-tt_fsi_status ttfsi_mg::masked_game_launch(const tt_fsi_mlp *model, const double *x_dev, const double *baseline_dev,
-                                           int64_t B, void *v_dev, int out_f32, double scale, int accumulate,
-                                           struct CUstream_st *stream) {
-    using namespace ttfsi_mg;
+// v = mean of f over the background rows (one row: the baseline).  Models of
+// up to 128 x 128 hidden units on at least 7 features take the split-digit
+// path on the tensor cores (masked_game_split.cu), one launch; others one
+// launch of masked_game_kernel per row, added in ascending order.
+static tt_fsi_status masked_game_launch(const tt_fsi_mlp *model, const double *x_dev, const double *bg_dev, int n_bg,
+                                        int64_t B, void *v_dev, int out_f32, struct CUstream_st *stream) {
     if (!model || B < 0) return TT_FSI_ERR_INVALID_ARG;
     if (B == 0) return TT_FSI_OK;
-    if (!x_dev || !baseline_dev || !v_dev || !model->W1 || !model->b1 || !model->W2 || !model->b2 ||
-        !model->W3)
+    if (!x_dev || !bg_dev || !v_dev || !model->W1 || !model->b1 || !model->W2 || !model->b2 || !model->W3)
         return TT_FSI_ERR_INVALID_ARG;
-    if (model->d < 1 || model->d > 30 || model->h1 < 1 || model->h2 < 1 || model->h1 > MAX_H ||
-        model->h2 > MAX_H)
+    if (model->d < 1 || model->d > 30 || model->h1 < 1 || model->h2 < 1 || model->h1 > MAX_H || model->h2 > MAX_H)
         return TT_FSI_ERR_INVALID_ARG;
     if (out_f32 && (!model->W2f || !model->b2f || !model->W3f)) return TT_FSI_ERR_INVALID_ARG;
-    Args a{model->W1, model->b1, model->W2, model->b2, model->W3, model->b3,
-           x_dev, baseline_dev, v_dev, model->d, model->h1, model->h2, 0,
-           model->W1f, model->b1f, model->W2f, model->b2f, model->W3f, scale, accumulate};
+    if (ttfsi_mgs::split_serves(model->d, model->h1, model->h2, out_f32))
+        return ttfsi_mgs::split_launch(model, x_dev, bg_dev, n_bg, B, v_dev, out_f32, stream);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const int g = model->d < G ? model->d : G;
     const size_t elem = out_f32 ? sizeof(float) : sizeof(double);
@@ -176,18 +157,39 @@ tt_fsi_status ttfsi_mg::masked_game_launch(const tt_fsi_mlp *model, const double
         e = cudaFuncSetAttribute(masked_game_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return TT_FSI_ERR_CUDA;
     const unsigned groups = 1u << (model->d - g);
-    for (int64_t g0 = 0; g0 < B; g0 += 65535) {
-        const unsigned nb = (unsigned)((B - g0) < 65535 ? (B - g0) : 65535);
-        a.game0 = g0;
-        dim3 grid(groups, nb);
-        if (out_f32)
-            masked_game_kernel<float><<<grid, THREADS, smem, st>>>(a);
-        else
-            masked_game_kernel<double><<<grid, THREADS, smem, st>>>(a);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? TT_FSI_ERR_NO_MEMORY : TT_FSI_ERR_CUDA;
+    const double scale = 1.0 / (double)n_bg;
+    for (int k = 0; k < n_bg; ++k) {
+        Args a{model->W1, model->b1, model->W2, model->b2, model->W3, model->b3,
+               x_dev, bg_dev + (size_t)k * model->d, v_dev, model->d, model->h1, model->h2, 0,
+               model->W1f, model->b1f, model->W2f, model->b2f, model->W3f, scale, k > 0};
+        for (int64_t g0 = 0; g0 < B; g0 += 65535) {
+            const unsigned nb = (unsigned)((B - g0) < 65535 ? (B - g0) : 65535);
+            a.game0 = g0;
+            dim3 grid(groups, nb);
+            if (out_f32)
+                masked_game_kernel<float><<<grid, THREADS, smem, st>>>(a);
+            else
+                masked_game_kernel<double><<<grid, THREADS, smem, st>>>(a);
+            e = cudaGetLastError();
+            if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? TT_FSI_ERR_NO_MEMORY : TT_FSI_ERR_CUDA;
+        }
     }
     return TT_FSI_OK;
+}
+
+}  // namespace ttfsi_mg
+
+extern "C" tt_fsi_status tt_fsi_masked_game(const tt_fsi_mlp *model, const double *x_dev,
+                                           const double *baseline_dev, int64_t B, void *v_dev,
+                                           int out_f32, struct CUstream_st *stream) {
+    return ttfsi_mg::masked_game_launch(model, x_dev, baseline_dev, 1, B, v_dev, out_f32, stream);
+}
+
+extern "C" tt_fsi_status tt_fsi_masked_game_interventional(const tt_fsi_mlp *model, const double *x_dev,
+                                                          const double *background_dev, int n_background, int64_t B,
+                                                          void *v_dev, int out_f32, struct CUstream_st *stream) {
+    if (!model || n_background < 1 || !background_dev) return TT_FSI_ERR_INVALID_ARG;
+    return ttfsi_mg::masked_game_launch(model, x_dev, background_dev, n_background, B, v_dev, out_f32, stream);
 }
 
 // ----------------------------------------------------------------------------
