@@ -476,6 +476,106 @@ __global__ void __launch_bounds__(32 * kC4Warps, 3) fsi_combine_split_kernel(Com
 }
 
 // ----------------------------------------------------------------------------
+// Small games of the exact fast path (d <= 11) in one launch: a warp forms one
+// score as the dot product of the game's fixed-point values with integer
+// coefficients that depend on (|S|, |R|, |S n R|) alone (see the plan), instead
+// of a 4096-wide tile padded with null players and a combine launch after it.
+// Both evaluate the same integer (the conversion, the denominator D_s and the
+// rounding at the end are the tile path's), so the scores are bitwise the same.
+// What bounds a single game is the chain launch - load - exponent - convert -
+// dot product; every CTA converts the whole game for its eight scores.
+// ----------------------------------------------------------------------------
+struct DirectArgs {
+    const unsigned long long *v;
+    double *phi;
+    int *err;
+    const int32_t *table;  // coefficients, then score masks
+    const double *winv;
+    int d, s1, n_coef, prec_bits;
+    long long n_out, game0;
+};
+
+constexpr int kDirectThreads = 256;
+constexpr int kDirectWarps = kDirectThreads / 32;
+constexpr int kDirectCoef = 5 * (kDirectMaxBits + 1) * 5;
+constexpr int kDirectLow = 21;  // low bits of a value, split for 32 x 32-bit products
+
+__global__ void __launch_bounds__(kDirectThreads) fsi_direct_kernel(DirectArgs a) {
+    __shared__ int2 val[1 << kDirectMaxBits];  // value >> kDirectLow, low bits
+    __shared__ int coef[kDirectCoef];
+    __shared__ int wmax[kDirectWarps];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, n = 1 << a.d;
+    const long long game = a.game0 + blockIdx.y;
+    const unsigned long long *src = a.v + (game << a.d);
+    constexpr int VPT = (1 << kDirectMaxBits) / kDirectThreads;
+    unsigned long long raw[VPT];
+    int emax = 0;
+#pragma unroll
+    for (int k = 0; k < VPT; ++k) {
+        const int e = tid + k * kDirectThreads;
+        raw[k] = e < n ? __ldg(src + e) : 0ull;
+        emax = max(emax, (int)((raw[k] >> 52) & 0x7ff));
+    }
+    const long long task = (long long)blockIdx.x * kDirectWarps + warp;
+    const bool active = task < a.n_out;
+    const unsigned S = active ? (unsigned)__ldg(a.table + a.n_coef + task) : 0u;
+    for (int i = tid; i < a.n_coef; i += kDirectThreads) coef[i] = __ldg(a.table + i);
+    emax = __reduce_max_sync(0xffffffffu, emax);
+    if (lane == 0) wmax[warp] = emax;
+    __syncthreads();
+    int E = wmax[0];
+#pragma unroll
+    for (int w = 1; w < kDirectWarps; ++w) E = max(E, wmax[w]);
+    // as the tile kernel's conversion
+    const bool bad = E == 0x7ff;
+    if (bad && tid == 0) atomicOr(a.err, kErrNonFinite);
+    if (E == 0) E = 1;
+    const int C = 53 - a.prec_bits + E;
+#pragma unroll
+    for (int k = 0; k < VPT; ++k) {
+        const int e = tid + k * kDirectThreads;
+        if (e >= n) break;
+        const long long x = bad ? 0ll : E >= a.prec_bits + 1 ? to_fixed_big_tile(raw[k], C) : to_fixed(raw[k], E, a.prec_bits);
+        val[e] = make_int2((int)(x >> kDirectLow), (int)(x & ((1 << kDirectLow) - 1)));
+    }
+    __syncthreads();
+    if (!active) return;
+    const int s = __popc(S);
+    const int *row = coef + s * (a.d + 1) * a.s1;
+    long long hi = 0, lo = 0;
+#pragma unroll 4
+    for (int R = lane; R < n; R += 32) {
+        const int c = row[__popc((unsigned)R) * a.s1 + __popc((unsigned)R & S)];
+        const int2 x = val[R];
+        hi += (long long)c * x.x;
+        lo += (long long)c * x.y;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        hi += __shfl_xor_sync(0xffffffffu, hi, o);
+        lo += __shfl_xor_sync(0xffffffffu, lo, o);
+    }
+    if (lane == 0) {
+        const int F = a.prec_bits + 1022 - E;
+        const __int128 acc = ((__int128)hi << kDirectLow) + lo;
+        double x, out;
+        if (i128_scaled_to_double(acc, F, x))
+            out = x * __ldg(a.winv + s);
+        else
+            out = ldexp(i128_to_double(acc) * __ldg(a.winv + s), -F);
+        a.phi[game * a.n_out + task] = out;
+    }
+}
+
+// Products (scores x values x games) of one call up to which the direct kernel
+// is taken.  Both measured (one GB300, us per call, direct against tiles +
+// combine): d = 8, l = 2: 4.1 / 10.3 for 1 to 32 games, 8.2 / 14.4 for 256;
+// d = 10, l = 3: 6.2 / 12.3 up to 16 games, 8.2 / 12.3 at 32 (2^22.5 products),
+// 14.4 / 12.3 at 64; d = 10, l = 2: 6.2 / 10.3, equal at 128 (2^22.8); d = 11,
+// l = 4: 8.2 / 14.4 at 4 games (2^22.1), 18.5 / 14.4 at 16.
+constexpr long long kDirectTerms = 3ll << 21;
+
+// ----------------------------------------------------------------------------
 // Fused apply of a fast-path plan: one persistent launch runs the tiles and
 // the combine of all B games.  Work items come from a device counter in the
 // order T(0), T(1), S(0), T(2), S(1), ..., T(B-1), S(B-2), S(B-1), where T(g)
@@ -727,7 +827,7 @@ struct TableRef {
     size_t bytes;
 };
 
-constexpr int kPlanTables = 9;
+constexpr int kPlanTables = 10;
 
 std::array<TableRef, kPlanTables> plan_tables(Plan &p) {
     return {{
@@ -740,6 +840,7 @@ std::array<TableRef, kPlanTables> plan_tables(Plan &p) {
         {(void **)&p.d_gtab, p.gtab.data(), p.gtab.size() * sizeof(int32_t)},
         {(void **)&p.d_wstage, p.wstage.data(), p.wstage.size()},
         {(void **)&p.d_winv, p.winv.data(), p.winv.size() * sizeof(double)},
+        {(void **)&p.d_direct, p.direct.data(), p.direct.size() * sizeof(int32_t)},
     }};
 }
 
@@ -768,6 +869,7 @@ void free_plan_device(Plan *p) {
     cudaFree(p->d_gtab);
     cudaFree(p->d_wstage);
     cudaFree(p->d_winv);
+    cudaFree(p->d_direct);
     cudaFree(p->d_counters);
 }
 
@@ -931,6 +1033,29 @@ tt_fsi_status launch_apply(const Plan &p, const void *v, int64_t B, void *phi, c
         if (ev1) cudaEventRecord(ev1, st);
         if (ev2) cudaEventRecord(ev2, st);
         return TT_FSI_OK;
+    }
+    if constexpr (TileTraits<Acc>::exact) {
+        if (p.fast12 && p.d_direct && B <= 65535 && ((p.n_out * B) << p.d) <= kDirectTerms) {
+            DirectArgs da{};
+            da.v = static_cast<const unsigned long long *>(v);
+            da.phi = static_cast<double *>(phi);
+            da.err = p.d_err;
+            da.table = p.d_direct;
+            da.winv = p.d_winv;
+            da.d = p.d;
+            da.s1 = p.ell_eff + 1;
+            da.n_coef = da.s1 * (p.d + 1) * da.s1;
+            da.prec_bits = p.prec_bits;
+            da.n_out = p.n_out;
+            if (ev0) cudaEventRecord(ev0, st);
+            const dim3 grid((unsigned)((p.n_out + kDirectWarps - 1) / kDirectWarps), (unsigned)B);
+            fsi_direct_kernel<<<grid, kDirectThreads, 0, st>>>(da);
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return cuda_status(e);
+            if (ev1) cudaEventRecord(ev1, st);
+            if (ev2) cudaEventRecord(ev2, st);
+            return TT_FSI_OK;
+        }
     }
     const int64_t chunk = 65535;
     for (int64_t g0 = 0; g0 < B; g0 += chunk) {

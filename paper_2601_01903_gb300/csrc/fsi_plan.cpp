@@ -496,6 +496,30 @@ tt_fsi_status plan_build_host(Plan &p, int d, int ell, tt_fsi_arith arith, int64
                         }
                     }
     }
+    // Direct coefficients of small games: phi(S) D_s = sum over T of S of c(|T|)
+    // a(T) with c(t) = W(s, t) D_s + [t = s] D_s, and a(T) = sum over R of T of
+    // (-1)^(|T| - |R|) v(R), so v(R) comes with the sum over T of S u R of
+    // c(|T|) (-1)^(|T| - |R|): C(d - u, n) sets T of size u + n, u = |S u R|.
+    p.direct.clear();
+    if (p.fast12 && arith == TT_FSI_ARITH_EXACT && d <= kDirectMaxBits) {
+        p.direct.assign((size_t)S1 * (d + 1) * S1, 0);
+        bool fits = true;
+        for (int s = 0; s < S1 && fits; ++s)
+            for (int r = 0; r <= d; ++r)
+                for (int i = 0; i <= std::min(s, r); ++i) {
+                    const int u = s + r - i;
+                    if (u > d) continue;
+                    __int128 sum = 0;
+                    for (int n = 0; n <= d - u; ++n) {
+                        const __int128 c = (__int128)p.wnum[(size_t)s * Q1 + u + n] + (u + n == s ? p.wden[s] : 0);
+                        sum += ((u + n - r) & 1 ? -c : c) * C(d - u, n);
+                    }
+                    fits = fits && iabs128(sum) < ((__int128)1 << 31);
+                    p.direct[((size_t)s * (d + 1) + r) * S1 + i] = (int32_t)sum;
+                }
+        for (int64_t i = 0; i < p.n_out; ++i) p.direct.push_back((int32_t)masks[i]);
+        if (!fits) p.direct.clear();
+    }
     return TT_FSI_OK;
 }
 

@@ -36,6 +36,8 @@ Rational weight_rational(int ell, int s, int t);
 // applied separately.
 Rational index_weight(tt_fsi_index index, int ell, int s, int t);
 
+constexpr int kDirectMaxBits = 11;
+
 struct Plan {
     bool precontract = false;  // site-by-site sweep of B_corr on v (no Moebius pass)
     int d = 0, ell = 0, ell_eff = 0;
@@ -90,6 +92,13 @@ struct Plan {
     std::vector<long long> wden;  // exact path: one common denominator per s
     std::vector<double> wf64;     // float paths
     std::vector<float> wf32;
+
+    // Small games of the exact fast path (d <= kDirectMaxBits, one tile): the
+    // coefficient of v(R) in phi(S) D_s depends on (|S|, |R|, |S n R|) only;
+    // [s][r][i] at (s (d + 1) + r) (l + 1) + i, then the n_out score masks.
+    // Empty where a coefficient does not fit in 32 bits.
+    std::vector<int32_t> direct;
+    int32_t *d_direct = nullptr;
 
     // device memory
     int32_t *d_trans = nullptr;
