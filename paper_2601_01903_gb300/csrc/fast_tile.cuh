@@ -584,14 +584,16 @@ __device__ __forceinline__ void tile_fast_body(const FastArgs &a, const long lon
     }
 }
 
-// One tile of a plan with order a.ell (1..4): the instantiation for that order.
-template <typename Acc>
+// One tile of a plan with order a.ell (1 .. MAXL): the instantiation for that order.
+template <typename Acc, int MAXL>
 __device__ __forceinline__ void tile_fast_dispatch(const FastArgs &a, const long long game, const long long tile) {
     switch (a.ell) {
         case 1: tile_fast_body<Acc, 1>(a, game, tile); break;
         case 2: tile_fast_body<Acc, 2>(a, game, tile); break;
         case 3: tile_fast_body<Acc, 3>(a, game, tile); break;
-        default: tile_fast_body<Acc, 4>(a, game, tile); break;
+        default:
+            if constexpr (MAXL > 3) tile_fast_body<Acc, 4>(a, game, tile);
+            break;
     }
 }
 

@@ -1624,6 +1624,15 @@ struct BatchItem {
     int game, first, count;  // tiles [first, first + count) or scores [first, first + count)
 };
 
+// CTAs per SM of the batch kernel, compiled for the highest order among a
+// batch's tiles (MAXL = 3 or 4).  Without order 4 (whose tiles need more
+// registers) and with an item's arguments in shared memory, the exact path fits
+// three CTAs in 80 registers (16 bytes spilled; 896 with every order and the
+// arguments in registers), float32 four.  1024 games of d 10 to 20: 1.71 ms at
+// two CTAs, 1.51 ms at three; 96 games: 0.190 and 0.162 ms.
+template <typename Acc, int MAXL>
+constexpr int kBatchMinBlocks = MAXL > 3 || sizeof(Acc) == 8 && !TileTraits<Acc>::exact ? 2 : TileTraits<Acc>::exact ? 3 : 4;
+
 struct BatchArgs {
     const void *v;
     void *phi;
@@ -1641,28 +1650,43 @@ struct BatchArgs {
     int inject_missing;  // test hook: every wait expects one tile more than exists
 };
 
-template <typename Acc>
-__global__ void __launch_bounds__(kTileThreads, 2) fsi_batch_kernel(BatchArgs a) {
+template <typename Acc, int MAXL>
+__global__ void __launch_bounds__(kTileThreads, kBatchMinBlocks<Acc, MAXL>) fsi_batch_kernel(BatchArgs a) {
     using GT = typename GTraits<Acc>::G;
     using In = typename TileTraits<Acc>::In;
     using Out = typename std::conditional<sizeof(Acc) == 4, float, double>::type;
+    // the item's arguments sit in shared memory, not in every thread's registers
     __shared__ int s_item, s_ok;
+    __shared__ FastArgs fa;
+    __shared__ CombineFastArgs ca;
+    __shared__ BatchItem it;
     for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(a.head, 1);
+        if (threadIdx.x == 0) {
+            const int k = atomicAdd(a.head, 1);
+            s_item = k;
+            if (k < a.n_items) {
+                it = a.items[k];
+                const BatchGameDev g = a.games[it.game];
+                if (k < a.n_tile_items) {
+                    fa = a.fplans[g.plan];
+                    fa.v = reinterpret_cast<const In *>(a.v) + g.v_off;
+                    fa.G = reinterpret_cast<GT *>(a.G) + g.g_off;
+                    fa.tile_exp = a.tile_exp + g.exp_off;
+                    fa.err = a.err;
+                } else {
+                    ca = a.cplans[g.plan];
+                    ca.G = reinterpret_cast<GT *>(a.G) + g.g_off;
+                    ca.tile_exp = a.tile_exp + g.exp_off;
+                    ca.phi = reinterpret_cast<Out *>(a.phi) + g.phi_off;
+                }
+            }
+        }
         __syncthreads();
         const int item = s_item;
-        __syncthreads();
         if (item >= a.n_items) break;
-        const BatchItem it = a.items[item];
-        const BatchGameDev g = a.games[it.game];
         if (item < a.n_tile_items) {
-            FastArgs fa = a.fplans[g.plan];
-            fa.v = reinterpret_cast<const In *>(a.v) + g.v_off;
-            fa.G = reinterpret_cast<GT *>(a.G) + g.g_off;
-            fa.tile_exp = a.tile_exp + g.exp_off;
-            fa.err = a.err;
             for (int t = it.first; t < it.first + it.count; ++t) {
-                tile_fast_dispatch<Acc>(fa, 0, t);
+                tile_fast_dispatch<Acc, MAXL>(fa, 0, t);
                 __syncthreads();
             }
             __threadfence();
@@ -1670,7 +1694,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) fsi_batch_kernel(BatchArgs a)
             if (threadIdx.x == 0) atomicAdd(a.done + it.game, it.count);
         } else {
             if (threadIdx.x == 0) {
-                const int need = g.n_tiles + (a.inject_missing ? 1 : 0);
+                const int need = a.games[it.game].n_tiles + (a.inject_missing ? 1 : 0);
                 int ok = 1;
                 long long polls = 0;
                 while (atomicAdd(a.done + it.game, 0) < need) {
@@ -1685,13 +1709,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) fsi_batch_kernel(BatchArgs a)
                 s_ok = ok;
             }
             __syncthreads();
-            if (s_ok) {
-                CombineFastArgs ca = a.cplans[g.plan];
-                ca.G = reinterpret_cast<GT *>(a.G) + g.g_off;
-                ca.tile_exp = a.tile_exp + g.exp_off;
-                ca.phi = reinterpret_cast<Out *>(a.phi) + g.phi_off;
-                combine_fast_body<Acc>(ca, 0, it.first, it.first + it.count);
-            }
+            if (s_ok) combine_fast_body<Acc>(ca, 0, it.first, it.first + it.count);
             __syncthreads();
         }
     }
@@ -1718,6 +1736,7 @@ struct tt_fsi_batch_s {
     void *d_G = nullptr;
     int *d_exp = nullptr;
     size_t smem = 0;
+    int max_ell = 1;  // highest order among the fast games
     int grid = 0;
     long long spin_limit = 4000000;
     int inject_missing = 0;
@@ -1759,6 +1778,15 @@ tt_fsi_status batch_build_items(tt_fsi_batch_s *b) {
     return cuda_status(e);
 }
 
+// Resident CTAs per SM of the batch kernel for these orders.
+template <typename Acc>
+cudaError_t batch_occupancy(int max_ell, size_t smem, int *occ) {
+    auto *kernel = max_ell <= 3 ? fsi_batch_kernel<Acc, 3> : fsi_batch_kernel<Acc, 4>;
+    cudaError_t e = allow_max_smem(kernel);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kernel, kTileThreads, smem);
+    return e;
+}
+
 void batch_free(tt_fsi_batch_s *b) {
     if (b->graph) cudaGraphExecDestroy(b->graph);
     if (b->graph_def) cudaGraphDestroy(b->graph_def);
@@ -1795,7 +1823,10 @@ tt_fsi_status batch_launch(tt_fsi_batch_s *b, const void *v, void *phi, cudaStre
         a.done = b->d_counters + 1;
         a.spin_limit = b->spin_limit;
         a.inject_missing = b->inject_missing;
-        fsi_batch_kernel<Acc><<<b->grid, kTileThreads, b->smem, st>>>(a);
+        if (b->max_ell <= 3)
+            fsi_batch_kernel<Acc, 3><<<b->grid, kTileThreads, b->smem, st>>>(a);
+        else
+            fsi_batch_kernel<Acc, 4><<<b->grid, kTileThreads, b->smem, st>>>(a);
         e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_status(e);
     }
@@ -1871,6 +1902,7 @@ tt_fsi_status tt_fsi_batch_create_index(const tt_fsi_game *games_host, int64_t n
             goff += (long long)hg.n_tiles * p.n_g;
             eoff += hg.n_tiles;
             b->smem = std::max(b->smem, p.smem_fast);
+            b->max_ell = std::max(b->max_ell, p.ell_eff);
         } else {
             b->slow_games.push_back((int)g);
         }
@@ -1908,16 +1940,12 @@ tt_fsi_status tt_fsi_batch_create_index(const tt_fsi_game *games_host, int64_t n
     if (e == cudaSuccess && eoff > 0) e = cudaMalloc((void **)&b->d_exp, (size_t)eoff * sizeof(int));
     if (e == cudaSuccess && !b->fast_games.empty()) {
         int occ = 0, dev = 0, sms = 0;
-        if (arith == TT_FSI_ARITH_EXACT) {
-            e = allow_max_smem(fsi_batch_kernel<long long>);
-            if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fsi_batch_kernel<long long>, kTileThreads, b->smem);
-        } else if (arith == TT_FSI_ARITH_F64) {
-            e = allow_max_smem(fsi_batch_kernel<double>);
-            if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fsi_batch_kernel<double>, kTileThreads, b->smem);
-        } else {
-            e = allow_max_smem(fsi_batch_kernel<float>);
-            if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fsi_batch_kernel<float>, kTileThreads, b->smem);
-        }
+        if (arith == TT_FSI_ARITH_EXACT)
+            e = batch_occupancy<long long>(b->max_ell, b->smem, &occ);
+        else if (arith == TT_FSI_ARITH_F64)
+            e = batch_occupancy<double>(b->max_ell, b->smem, &occ);
+        else
+            e = batch_occupancy<float>(b->max_ell, b->smem, &occ);
         if (e == cudaSuccess) e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         b->grid = std::max(1, occ) * sms;  // every CTA resident at once: waits can always be served
