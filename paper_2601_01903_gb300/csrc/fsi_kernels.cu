@@ -224,6 +224,29 @@ __device__ __forceinline__ bool i128_scaled_to_double(__int128 x, int F, double 
     return true;
 }
 
+// The float paths add a score's partial scores in segments of tiles: one
+// segment below 1024 tiles, else one per warp of a CTA.
+__device__ __forceinline__ int combine_segments(int ntile) { return ntile < 1024 ? 1 : kCombineFastWarps; }
+
+// Lane sums of tiles [u_begin, u_begin + len) of one score.
+template <typename Acc>
+__device__ __forceinline__ Acc combine_segment(const Acc *Gs, unsigned SH, int ntile, int u_begin, int len, int lane) {
+    constexpr int U = 8;  // independent loads in flight per lane
+    const int u_end = u_begin + len;
+    Acc acc = 0;
+    for (int u0 = u_begin + lane; u0 < u_end; u0 += 32 * U) {
+        Acc part[U];
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            const int u = u0 + 32 * k;
+            part[k] = (u < u_end) ? __ldcg(Gs + (long long)__popc((unsigned)u & SH) * ntile + u) : (Acc)0;
+        }
+#pragma unroll
+        for (int k = 0; k < U; ++k) acc += part[k];
+    }
+    return acc;
+}
+
 // Scores [task_begin, task_end) of one game; warp w takes task_begin + w,
 // + kCombineFastWarps, ...  Partial scores are read past L1 (ld.global.cg):
 // in the persistent batch kernel other CTAs wrote them during this launch.
@@ -316,25 +339,42 @@ __device__ __forceinline__ void combine_fast_body(const CombineFastArgs &a, cons
             }
         }
     } else {
-        constexpr int U = 8;
         for (long long task = task_begin + warp; task < task_end; task += kCombineFastWarps) {
             const unsigned SH = (unsigned)a.tasks[task * 4 + 1];
             const GT *Gs = Gg + (long long)a.tasks[task * 4 + 3] * ntile;
+            const int n_seg = combine_segments(ntile), len = ntile / n_seg;
             Acc acc = 0;
-            for (int u0 = lane; u0 < ntile; u0 += 32 * U) {
-                Acc part[U];
-#pragma unroll
-                for (int k = 0; k < U; ++k) {
-                    const int u = u0 + 32 * k;
-                    part[k] = (u < ntile) ? __ldcg(Gs + (long long)__popc((unsigned)u & SH) * ntile + u) : (Acc)0;
-                }
-#pragma unroll
-                for (int k = 0; k < U; ++k) acc += part[k];
-            }
+            for (int k = 0; k < n_seg; ++k) acc += combine_segment<Acc>(Gs, SH, ntile, k * len, len, lane);
             for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
             if (lane == 0) reinterpret_cast<Acc *>(a.phi)[game * a.n_out + task] = acc;
         }
     }
+}
+
+// Float paths, games of many tiles (combine_segments > 1): a CTA per score, a
+// warp per segment, the segments' lane sums added in segment order (the same
+// sums as combine_fast_body's, so that both schedules agree bit for bit).  One
+// warp per score leaves 38 CTAs with a chain of 128 loads per lane at d = 24,
+// l = 2; here every SM has two CTAs with chains of 16 (float32 call 55.5 -> 49.3
+// us; d = 22, l = 2 18.6 -> 17.3).
+template <typename Acc>
+__global__ void __launch_bounds__(32 * kCombineFastWarps) fsi_combine_wide_kernel(CombineFastArgs a) {
+    static_assert(!TileTraits<Acc>::exact, "float arithmetics");
+    __shared__ Acc red[kCombineFastWarps][32];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, ntile = 1 << a.h, len = ntile / kCombineFastWarps;
+    const long long game = a.game0 + blockIdx.y, task = blockIdx.x;
+    const unsigned SH = (unsigned)__ldg(a.tasks + task * 4 + 1);
+    const Acc *Gs = reinterpret_cast<const Acc *>(a.G) + (game << a.h) * (long long)a.n_g +
+                    (long long)__ldg(a.tasks + task * 4 + 3) * ntile;
+    red[warp][lane] = combine_segment<Acc>(Gs, SH, ntile, warp * len, len, lane);
+    __syncthreads();
+    if (warp) return;
+    Acc acc = 0;
+#pragma unroll
+    for (int k = 0; k < kCombineFastWarps; ++k) acc += red[k][lane];
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if (lane == 0) reinterpret_cast<Acc *>(a.phi)[game * a.n_out + task] = acc;
 }
 
 template <typename Acc>
@@ -349,11 +389,10 @@ __global__ void __launch_bounds__(32 * kCombineFastWarps) fsi_combine_fast_kerne
 
 // ----------------------------------------------------------------------------
 // Combine of the split schedule for games of at most 2^12 tiles (exact
-// arithmetic): kC4Lanes lanes per score, each summing every kC4Lanes-th tile
-// (so the lanes of a score read consecutive partial scores), 32 / kC4Lanes
-// scores per warp.  Compared with one warp per score, each lane sums
-// 2^h / kC4Lanes terms in registers and the cross-lane reduction is three
-// shuffle steps, not five; the first batch of partial-score loads is issued
+// arithmetic): QL lanes per score, each summing every QL-th tile (so the lanes
+// of a score read consecutive partial scores).  Compared with one warp per
+// score, at QL = 8 each lane sums 2^h / 8 terms in registers and the cross-lane
+// reduction is three shuffle steps, not five; the first batch of partial-score loads is issued
 // before the game's exponent range is known, so the exponent pass overlaps
 // it; the tiles' alignment shifts are computed once per CTA into shared
 // memory and skipped when all tiles of the game share one exponent.  Partial
@@ -362,9 +401,14 @@ __global__ void __launch_bounds__(32 * kCombineFastWarps) fsi_combine_fast_kerne
 // score routine (its rounding right shifts).
 // ----------------------------------------------------------------------------
 constexpr int kC4Warps = 8;
-constexpr int kC4Lanes = 8;                                // lanes per score
-constexpr int kC4Scores = kC4Warps * (32 / kC4Lanes);     // scores per CTA
-constexpr int kC4MaxTiles = 4096;                          // h <= 12: per-tile shifts in shared memory
+constexpr int kC4MaxTiles = 4096;  // h <= 12: per-tile shifts in shared memory
+
+// Lanes per score, QL = 8, 32, or the whole CTA (256): few scores over many
+// tiles (d = 24, l = 2: 301 scores, 4096 tiles) would leave most SMs idle with
+// long chains of loads at 8.  The sums are exact, so any split gives the same
+// integers.
+template <int QL>
+constexpr int kC4Scores = 32 * kC4Warps / QL;  // scores per CTA
 
 __device__ __forceinline__ __int128 shfl_xor_i128(__int128 v, int o) {
     unsigned long long lo = (unsigned long long)v, hi = (unsigned long long)((unsigned __int128)v >> 64);
@@ -373,24 +417,25 @@ __device__ __forceinline__ __int128 shfl_xor_i128(__int128 v, int o) {
     return (__int128)(((unsigned __int128)hi << 64) | lo);
 }
 
-template <typename Acc>
+template <typename Acc, int QL>
 __global__ void __launch_bounds__(32 * kC4Warps, 3) fsi_combine_split_kernel(CombineFastArgs a) {
     static_assert(TileTraits<Acc>::exact, "exact arithmetic only");
     using GT = typename GTraits<Acc>::G;
     constexpr int U = 8;  // partial-score loads in flight per lane
+    constexpr int kScores = kC4Scores<QL>;
     // launched as the tile grid's programmatic dependent: wait until that
     // grid has finished and its partial scores and exponents are visible
     // (returns at once otherwise); they are read past L1 (ld.global.cg)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     __shared__ unsigned char s_shift[kC4MaxTiles];
-    __shared__ int s_f[kC4MaxTiles];  // the game's tile exponents
+    __shared__ __align__(16) int s_f[kC4MaxTiles];  // the game's tile exponents
     __shared__ int s_fmin, s_fmax;
     const long long game = a.game0 + blockIdx.y;
     const int ntile = 1 << a.h;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = lane % kC4Lanes;
-    const long long t_begin = (long long)blockIdx.x * kC4Scores;
-    const long long t_end = t_begin + kC4Scores < a.n_out ? t_begin + kC4Scores : a.n_out;
-    const long long task = t_begin + warp * (32 / kC4Lanes) + lane / kC4Lanes;
+    const int lane = threadIdx.x & 31, q = threadIdx.x % QL;
+    const long long t_begin = (long long)blockIdx.x * kScores;
+    const long long t_end = t_begin + kScores < a.n_out ? t_begin + kScores : a.n_out;
+    const long long task = t_begin + threadIdx.x / QL;
     const bool active = task < t_end;
     // lanes past the last score stay for the shuffles but sum nothing
     const long long tk = active ? task : t_begin;
@@ -402,7 +447,7 @@ __global__ void __launch_bounds__(32 * kC4Warps, 3) fsi_combine_split_kernel(Com
     auto load_batch = [&](int u0, longlong2 (&raw)[U]) {
 #pragma unroll
         for (int k = 0; k < U; ++k) {
-            const int u = u0 + kC4Lanes * k;
+            const int u = u0 + QL * k;
             raw[k] = u < ntile ? __ldcg(reinterpret_cast<const longlong2 *>(
                                      row + (long long)__popc((unsigned)u & SH) * ntile + u))
                                : make_longlong2(0, 0);
@@ -451,19 +496,28 @@ __global__ void __launch_bounds__(32 * kC4Warps, 3) fsi_combine_split_kernel(Com
             const unsigned long long lo = (unsigned long long)raw[k].x;
             unsigned long long hi = (unsigned long long)raw[k].y, l2 = lo;
             if (shifts) {
-                const int u = u0 + kC4Lanes * k;
+                const int u = u0 + QL * k;
                 const int delta = u < ntile ? s_shift[u] : 0;
                 hi = (hi << delta) | ((lo >> 1) >> (63 - delta));
                 l2 = lo << delta;
             }
             acc += (__int128)(((unsigned __int128)hi << 64) | l2);
         }
-        u0 += kC4Lanes * U;
+        u0 += QL * U;
         if (u0 >= ntile) break;
         load_batch(u0, raw);
     }
 #pragma unroll
-    for (int o = 1; o < kC4Lanes; o <<= 1) acc += shfl_xor_i128(acc, o);
+    for (int o = 1; o < (QL < 32 ? QL : 32); o <<= 1) acc += shfl_xor_i128(acc, o);
+    if constexpr (QL > 32) {  // one score per CTA: the warps' sums
+        longlong2 *red = reinterpret_cast<longlong2 *>(s_f);  // the exponents have been used
+        __syncthreads();
+        if (lane == 0) red[threadIdx.x >> 5] = make_longlong2((long long)acc, (long long)(acc >> 64));
+        __syncthreads();
+        acc = 0;
+        for (int w = 0; w < kC4Warps; ++w)
+            acc += (__int128)(((unsigned __int128)(unsigned long long)red[w].y << 64) | (unsigned long long)red[w].x);
+    }
     if (active && q == 0) {
         // phi = acc 2^-Fc / D_s (see combine_fast_body)
         double x, out;
@@ -1110,8 +1164,17 @@ tt_fsi_status launch_apply(const Plan &p, const void *v, int64_t B, void *phi, c
             // fused schedule)
             if constexpr (TileTraits<Acc>::exact) {
                 if (p.h <= 12) {
-                    dim3 g2((unsigned)((p.n_out + kC4Scores - 1) / kC4Scores), (unsigned)nb);
-                    cudaError_t le = launch_dependent(fsi_combine_split_kernel<Acc>, g2, dim3(32 * kC4Warps), st, cf);
+                    // the fewest lanes per score that give every SM two CTAs, at
+                    // least one batch of loads per lane (us per call at 8 lanes and
+                    // now: d = 24, l = 2, one game 133.5 / 94.4; l = 1 109.1 / 69.8;
+                    // d = 22, l = 3 57.2 / 47.3; d = 20, l = 3 19.0 / 16.6)
+                    const int64_t want = 2 * 152 * 32 * kC4Warps, scores = p.n_out * nb;
+                    const int ql = scores * 8 >= want || p.h < 8 ? 8 : scores * 32 >= want || p.h < 11 ? 32 : 256;
+                    const int per = 32 * kC4Warps / ql;
+                    dim3 g2((unsigned)((p.n_out + per - 1) / per), (unsigned)nb);
+                    auto *kernel = ql == 8 ? fsi_combine_split_kernel<Acc, 8>
+                                           : ql == 32 ? fsi_combine_split_kernel<Acc, 32> : fsi_combine_split_kernel<Acc, 256>;
+                    cudaError_t le = launch_dependent(kernel, g2, dim3(32 * kC4Warps), st, cf);
                     if (le != cudaSuccess) return cuda_status(le);
                 } else {
                     dim3 g2((unsigned)((p.n_out + kCombineFastWarps - 1) / kCombineFastWarps), (unsigned)nb);
@@ -1119,8 +1182,10 @@ tt_fsi_status launch_apply(const Plan &p, const void *v, int64_t B, void *phi, c
                     if (le != cudaSuccess) return cuda_status(le);
                 }
             } else {
-                dim3 g2((unsigned)((p.n_out + kCombineFastWarps - 1) / kCombineFastWarps), (unsigned)nb);
-                cudaError_t le = launch_dependent(fsi_combine_fast_kernel<Acc>, g2, dim3(32 * kCombineFastWarps), st, cf);
+                const bool wide = p.h >= 10;  // combine_segments
+                dim3 g2((unsigned)(wide ? p.n_out : (p.n_out + kCombineFastWarps - 1) / kCombineFastWarps), (unsigned)nb);
+                cudaError_t le = launch_dependent(wide ? fsi_combine_wide_kernel<Acc> : fsi_combine_fast_kernel<Acc>, g2,
+                                                  dim3(32 * kCombineFastWarps), st, cf);
                 if (le != cudaSuccess) return cuda_status(le);
             }
         } else {
