@@ -5,8 +5,7 @@
 //
 //   C[M, N] = A[M, K] . B[N, K]^T      (both operands K-major, row-major in HBM)
 //
-// One CTA (4 warps) computes a 128 x BN tile (of one K slice when K is
-// split over the grid's third dimension).  Operand tiles of 128 x 64
+// One CTA (4 warps) computes a 128 x BN tile.  Operand tiles of 128 x 64
 // bf16 are staged in shared memory in the 128-byte swizzled K-major layout
 // (row r at r * 128 bytes, its 16-byte chunk c at chunk c ^ (r & 7)), two
 // stages deep: cp.async fills stage s + 1 while the tensor cores read stage
@@ -53,11 +52,6 @@ struct GemmArgs {
     __nv_bfloat16 *Ct;         // BF16 result transposed ([N, M]), or null
     int ldct;
     int *err;
-    // split K: CTA z of the grid's third dimension takes K blocks
-    // [z kbc, (z + 1) kbc) and writes its raw FP32 partial product to
-    // Cf + z cf_zstride (only Cf; the caller adds the slices); kbc = 0: all of K
-    int kbc;
-    long long cf_zstride;
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -168,7 +162,7 @@ __device__ __forceinline__ void load_tile(uint32_t tile, const __nv_bfloat16 *G,
 // `stage_all` is idle shared memory, 32 x 33 floats per warp; `slot` picks
 // the warp's block, the warp reads TMEM lane quarter `quarter` (tile rows
 // 32 quarter ..) over accumulator columns [cb, ce).
-__device__ __forceinline__ void gemm_epilogue(const GemmArgs &a, float *Cf, uint32_t tmem, float *stage_all, int m0,
+__device__ __forceinline__ void gemm_epilogue(const GemmArgs &a, uint32_t tmem, float *stage_all, int m0,
                                               int n0, int slot, int quarter, int cb, int ce, int lane) {
         float *stage = stage_all + slot * (32 * 33);
         // Epilogue, 32 columns at a time.  Warp w owns accumulator rows
@@ -219,7 +213,7 @@ __device__ __forceinline__ void gemm_epilogue(const GemmArgs &a, float *Cf, uint
                     if (row < a.M && col_ok) {
                         float z = stage[(i0 + i) * 33 + lane] + bias;
                         if (a.dgelu_z) z *= gelu_grad_f(zin[i]);
-                        if (Cf) Cf[(long long)row * a.ldcf + col] = z;
+                        if (a.Cf) a.Cf[(long long)row * a.ldcf + col] = z;
                         const float y = (a.act == 1) ? gelu_f(z) : z;
                         if (a.Cb) a.Cb[(long long)row * a.ldcb + col] = __float2bfloat16_rn(y);
                         stage[(i0 + i) * 33 + lane] = y;
@@ -251,10 +245,7 @@ __global__ void __launch_bounds__(THREADS) gemm_bf16_tcgen05(GemmArgs a) {
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-    const int nk_all = (a.K + BK - 1) / BK;
-    const int kb0 = a.kbc > 0 ? (int)blockIdx.z * a.kbc : 0;
-    const int nk = a.kbc > 0 ? min(a.kbc, nk_all - kb0) : nk_all;  // K blocks of this CTA
-    float *const Cf = a.Cf ? a.Cf + (long long)blockIdx.z * a.cf_zstride : nullptr;
+    const int nk = (a.K + BK - 1) / BK;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) mbar_init(smem_u32(&mbar[s]), 1);
@@ -278,8 +269,8 @@ __global__ void __launch_bounds__(THREADS) gemm_bf16_tcgen05(GemmArgs a) {
     bool fail = false;
 
     // prologue: stage 0
-    load_tile(tileA(0), a.A, a.lda, m0, a.M, kb0 * BK, a.K);
-    load_tile(tileB(0), a.B, a.ldb, n0, a.N, kb0 * BK, a.K);
+    load_tile(tileA(0), a.A, a.lda, m0, a.M, 0, a.K);
+    load_tile(tileB(0), a.B, a.ldb, n0, a.N, 0, a.K);
     asm volatile("cp.async.commit_group;" ::: "memory");
 
     for (int kb = 0; kb < nk && !fail; ++kb) {
@@ -292,8 +283,8 @@ __global__ void __launch_bounds__(THREADS) gemm_bf16_tcgen05(GemmArgs a) {
                 issued_bits &= ~(1u << sn);
             }
             if (!fail) {
-                load_tile(tileA(sn), a.A, a.lda, m0, a.M, (kb0 + kb + 1) * BK, a.K);
-                load_tile(tileB(sn), a.B, a.ldb, n0, a.N, (kb0 + kb + 1) * BK, a.K);
+                load_tile(tileA(sn), a.A, a.lda, m0, a.M, (kb + 1) * BK, a.K);
+                load_tile(tileB(sn), a.B, a.ldb, n0, a.N, (kb + 1) * BK, a.K);
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
             asm volatile("cp.async.wait_group 1;" ::: "memory");
@@ -307,7 +298,7 @@ __global__ void __launch_bounds__(THREADS) gemm_bf16_tcgen05(GemmArgs a) {
         if (fail) break;
         if (threadIdx.x == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int kmax = min(BK, a.K - (kb0 + kb) * BK);
+            const int kmax = min(BK, a.K - kb * BK);
             for (int k16 = 0; k16 * 16 < kmax; ++k16) {
                 const uint64_t da = smem_desc(tileA(s) + k16 * 32);
                 const uint64_t db = smem_desc(tileB(s) + k16 * 32);
@@ -328,7 +319,7 @@ __global__ void __launch_bounds__(THREADS) gemm_bf16_tcgen05(GemmArgs a) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
     if (!s_fail) {
-        gemm_epilogue(a, Cf, tmem, reinterpret_cast<float *>(gsm_raw + (base - raw)), m0, n0, warp, warp, 0, BN, lane);
+        gemm_epilogue(a, tmem, reinterpret_cast<float *>(gsm_raw + (base - raw)), m0, n0, warp, warp, 0, BN, lane);
     } else if (threadIdx.x == 0) {
         atomicOr(a.err, kErrGemmTimeout);
     }
@@ -377,10 +368,7 @@ __global__ void __launch_bounds__(TMA_THREADS) gemm_bf16_tcgen05_tma(const __gri
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-    const int nk_all = (a.K + BK - 1) / BK;
-    const int kb0 = a.kbc > 0 ? (int)blockIdx.z * a.kbc : 0;
-    const int nk = a.kbc > 0 ? min(a.kbc, nk_all - kb0) : nk_all;
-    float *const Cf = a.Cf ? a.Cf + (long long)blockIdx.z * a.cf_zstride : nullptr;
+    const int nk = (a.K + BK - 1) / BK;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < TMA_STAGES; ++s) {
@@ -418,7 +406,7 @@ __global__ void __launch_bounds__(TMA_THREADS) gemm_bf16_tcgen05_tma(const __gri
             }
             if (*(volatile int *)&s_fail) break;
             mbar_expect_tx(smem_u32(&full[s]), 2u * TILE_BYTES);
-            const int k0 = (kb0 + kb) * BK;
+            const int k0 = kb * BK;
             tma_load_2d(tileA(s), &tmA, k0, m0, smem_u32(&full[s]));
             tma_load_2d(tileB(s), &tmB, k0, n0, smem_u32(&full[s]));
         }
@@ -461,7 +449,7 @@ __global__ void __launch_bounds__(TMA_THREADS) gemm_bf16_tcgen05_tma(const __gri
         // the stage buffers are idle: every load was consumed by an MMA that has completed
         // 8 warps: warps w and w + 4 share TMEM lane quarter w & 3 and take
         // the accumulator columns [0, BN/2) and [BN/2, BN)
-        gemm_epilogue(a, Cf, tmem, reinterpret_cast<float *>(gsm_raw + (base - raw)), m0, n0, warp, warp & 3,
+        gemm_epilogue(a, tmem, reinterpret_cast<float *>(gsm_raw + (base - raw)), m0, n0, warp, warp & 3,
                       (warp >> 2) * (BN / 2), (warp >> 2) * (BN / 2) + BN / 2, lane);
     } else if (threadIdx.x == 0) {
         atomicOr(a.err, kErrGemmTimeout);

@@ -10,6 +10,7 @@
 #include <algorithm>
 
 #include "gemm_tcgen05.cuh"
+#include "student_gemm.cuh"
 #include "tt_fsi.h"
 
 namespace {
@@ -67,39 +68,13 @@ tt_fsi_status gemm_launch(const ttfsi_gemm::GemmArgs &a, cudaStream_t st) {
         if (e != cudaSuccess) return st_status(e);
         g_gemm_attr_set[dev] = true;
     }
-    const int nk = (a.K + BK - 1) / BK;
-    const int kslices = a.kbc > 0 ? (nk + a.kbc - 1) / a.kbc : 1;
-    dim3 grid((unsigned)((a.N + BN - 1) / BN), (unsigned)((a.M + BM - 1) / BM), (unsigned)kslices);
+    dim3 grid((unsigned)((a.N + BN - 1) / BN), (unsigned)((a.M + BM - 1) / BM));
     CUtensorMap tmA, tmB;
     if (operand_tensor_map(&tmA, a.A, a.M, a.K, a.lda) && operand_tensor_map(&tmB, a.B, a.N, a.K, a.ldb))
         gemm_bf16_tcgen05_tma<<<grid, TMA_THREADS, TMA_SMEM_BYTES, st>>>(a, tmA, tmB);
     else
         gemm_bf16_tcgen05<<<grid, THREADS, SMEM_BYTES, st>>>(a);
     return st_status(cudaGetLastError());
-}
-
-// Sum of the K-slice partial products in slice order, plus an optional bias
-// per column: C[r, c] = sum_z P_z[r, c] (+ bias[c]).
-__global__ void ksum_kernel(const float *part, long long zstride, int slices, int M, int N, int ld, const float *bias,
-                            float *C) {
-    const long long n = (long long)M * N;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const long long r = i / N, c = i - r * N;
-        float s = 0.f;
-        for (int z = 0; z < slices; ++z) s += part[z * zstride + r * ld + c];
-        C[r * ld + c] = bias ? s + bias[c] : s;
-    }
-}
-
-// K blocks per slice for a plain (Cf-only) product: split K when the output
-// tiles alone cannot fill the GPU, keeping at least 4 K blocks per slice.
-int split_kbc(int M, int N, int K) {
-    const int tiles = ((M + ttfsi_gemm::BM - 1) / ttfsi_gemm::BM) * ((N + ttfsi_gemm::BN - 1) / ttfsi_gemm::BN);
-    const int nk = (K + ttfsi_gemm::BK - 1) / ttfsi_gemm::BK;
-    if (tiles >= 128 || nk < 8) return 0;
-    int slices = std::min((2 * 152 + tiles - 1) / tiles, nk / 4);
-    if (slices < 2) return 0;
-    return (nk + slices - 1) / slices;
 }
 
 }  // namespace
@@ -140,174 +115,236 @@ extern "C" tt_fsi_status tt_fsi_gemm_bf16(const void *A, int lda, const void *B,
 // efficiency constraint.
 // ============================================================================
 #include <cmath>
+#include <cstring>
 #include <new>
+#include <utility>
 #include <vector>
 
 namespace ttfsi_student {
 
 using bf16 = __nv_bfloat16;
-constexpr int kErrTimeout = 1;
 
-// FP32 [rows, cols] (row-major) -> BF16 copy Wb [rows_pad, cols] (rows >= rows
-// zero; optional) and transposed BF16 copy Wt [cols, ldt] with Wt[c][r] =
-// W[r][c] for r < rows_pad (zero for r >= rows; optional), through 32 x 32
-// shared-memory tiles so that the reads and both writes are coalesced.
-// Block 32 x 8 threads, grid (ceil(cols / 32), ceil(rows_pad / 32)).
-__device__ __forceinline__ void to_bf16_tile(const float *W, int rows, int cols, int rows_pad, bf16 *Wb, bf16 *Wt,
-                                             int ldt, int c0, int r0) {
-    __shared__ float tile[32][33];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    for (int i = ty; i < 32; i += 8) {
-        const int r = r0 + i, c = c0 + tx;
-        const float w = (r < rows && c < cols) ? W[(long long)r * cols + c] : 0.0f;
-        tile[i][tx] = w;
-        if (Wb && r < rows_pad && c < cols) Wb[(long long)r * cols + c] = __float2bfloat16_rn(w);
-    }
-    if (!Wt) return;
-    __syncthreads();
-    for (int i = ty; i < 32; i += 8) {
-        const int c = c0 + i, r = r0 + tx;
-        if (c < cols && r < rows_pad) Wt[(long long)c * ldt + r] = __float2bfloat16_rn(tile[tx][i]);
-    }
-}
-
-__global__ void to_bf16_tiled_kernel(const float *W, int rows, int cols, int rows_pad, bf16 *Wb, bf16 *Wt, int ldt) {
-    to_bf16_tile(W, rows, cols, rows_pad, Wb, Wt, ldt, blockIdx.x * 32, blockIdx.y * 32);
-}
-
-// Several casts in one launch: block b takes tile b - first[j] of cast j
-// (the casts' tiles are numbered one after another, column tiles fastest).
-struct CastJob {
-    const float *W;
-    bf16 *Wb, *Wt;
-    int rows, cols, rows_pad, ldt, tiles_x, first;
-};
+// BF16 copies of up to three FP32 arrays (the weights on load, a batch of
+// instances), one launch: element i of the concatenation.
 struct CastJobs {
-    CastJob j[3];
-    int n;
+    const float *src[3];
+    bf16 *dst[3];
+    long long n[3];
 };
-__global__ void to_bf16_multi_kernel(CastJobs jobs) {
-    int k = 0;
-    while (k + 1 < jobs.n && (int)blockIdx.x >= jobs.j[k + 1].first) ++k;
-    const CastJob &c = jobs.j[k];
-    const int t = (int)blockIdx.x - c.first;
-    to_bf16_tile(c.W, c.rows, c.cols, c.rows_pad, c.Wb, c.Wt, c.ldt, (t % c.tiles_x) * 32, (t / c.tiles_x) * 32);
+__global__ void to_bf16_kernel(CastJobs c) {
+    ttfsi_sgemm::pdl_launch();
+    ttfsi_sgemm::pdl_wait();
+    const long long step = (long long)gridDim.x * blockDim.x;
+    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    for (int k = 0; k < 3; ++k) {
+        for (; i < c.n[k]; i += step) c.dst[k][i] = __float2bfloat16_rn(c.src[k][i]);
+        i -= c.n[k];
+    }
 }
 
-// Projection onto sum_{S != empty} phi(S) = target, phi(empty) = v_empty, then
-// (if labels are given) the squared-error loss and its gradient with respect
-// to the raw outputs: dL/dY = P (2 (phi_p - phi) / (B n_out)), P = I - 11^T/(n_out-1)
-// on the non-empty coordinates, 0 on the empty one.  One warp per instance.
-__global__ void project_loss_kernel(const float *Y, int B, int n_out, const float *target, float v_empty, float *phi,
-                                    const float *labels, float *loss_rows, float *dYf, bf16 *dYb, int ld_dyb, bf16 *dYt,
-                                    int ld_dyt) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (warp >= B) return;
-    const float *y = Y + (long long)warp * n_out;
-    float s = 0.f;
-    for (int k = 1 + lane; k < n_out; k += 32) s += y[k];
+// Output layer and projection onto sum_{S != empty} phi(S) = target,
+// phi(empty) = v_empty: y = the K slices of A2 W3^T added in order, plus b3.
+// With labels also the squared-error loss and its gradient with respect to the
+// raw outputs, dL/dY = P (2 (phi_p - phi) / (B n_out)), P = I - 11^T/(n_out-1)
+// on the non-empty coordinates, 0 on the empty one, as BF16 (the operand of
+// the backward products), its FP32 column sums over the block's rows (the bias
+// gradient's partial sums) and the block's loss.  A warp takes R rows, a block
+// 8 R; y is kept in the first slice's row, which only its own lanes read.
+struct ProjectArgs {
+    float *Y;  // [slices][zrows][ldy]
+    int slices, ldy;
+    long long zstride;
+    const float *bias;
+    int B, n_out;
+    const float *target;
+    float v_empty;
+    float *phi;           // [B, n_out], or null
+    const float *labels;  // [B, n_out], or null: no loss, no gradient
+    float *loss_part, *col_part;  // [blocks], [blocks][n_out]
+    bf16 *dYb;
+    int ld_dyb;
+};
+
+__device__ __forceinline__ float warp_sum(float s) {
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    const float shift = (target[warp] - s) / (float)(n_out - 1);
-    float loss = 0.f, gsum = 0.f;
-    const float scale = 2.0f / ((float)B * (float)n_out);
-    for (int k = lane; k < n_out; k += 32) {
-        const float p = (k == 0) ? v_empty : y[k] + shift;
-        if (phi) phi[(long long)warp * n_out + k] = p;
-        if (labels) {
-            const float e = p - labels[(long long)warp * n_out + k];
-            loss += e * e;
-            if (k > 0) gsum += scale * e;
-        }
-    }
-    if (!labels) return;
-    for (int o = 16; o > 0; o >>= 1) {
-        loss += __shfl_xor_sync(0xffffffffu, loss, o);
-        gsum += __shfl_xor_sync(0xffffffffu, gsum, o);
-    }
-    if (lane == 0) loss_rows[warp] = loss;
-    const float gmean = gsum / (float)(n_out - 1);
-    for (int k = lane; k < ld_dyb; k += 32) {
-        float g = 0.f;
-        if (k > 0 && k < n_out) {
-            const float p = y[k] + shift;
-            g = scale * (p - labels[(long long)warp * n_out + k]) - gmean;
-        }
-        if (k < n_out) dYf[(long long)warp * n_out + k] = g;
-        const bf16 gb = __float2bfloat16_rn(g);
-        dYb[(long long)warp * ld_dyb + k] = gb;
-        if (dYt && k < n_out) dYt[(long long)k * ld_dyt + warp] = gb;
-    }
+    return s;
 }
 
-// Column sums of an FP32 [M, N] matrix in a fixed order, one launch.  Block
-// (32 columns, a slab of 256 rows), 32 x 8 threads; thread (x, y) sums rows
-// 32y..32y+31 of the slab, the 8 partials are added in order and written to
-// part[slab][N].  The last block to finish a column block (an arrival
-// counter per column block, reset by that block for the next call) adds the
-// slab partials of its 32 columns in slab order.  No block waits for
-// another.
-__global__ void colsum_kernel(const float *X, int M, int N, float *part, int *arrivals, float *out) {
-    __shared__ float red[8][33];
-    __shared__ int s_last;
-    const int c = blockIdx.x * 32 + threadIdx.x;
-    const int r0 = blockIdx.y * 256 + threadIdx.y * 32;
-    float s = 0.f;
-    if (c < N) {
-        const int r1 = min(r0 + 32, M);
-        for (int r = r0; r < r1; ++r) s += X[(long long)r * N + c];
-    }
-    red[threadIdx.y][threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.y == 0) {
-        if (c < N) {
-            float t = 0.f;
-            for (int k = 0; k < 8; ++k) t += red[k][threadIdx.x];
-            part[(long long)blockIdx.y * N + c] = t;
+template <int R>
+__global__ void __launch_bounds__(256) project_kernel(const ProjectArgs a) {
+    __shared__ float red[8][32];
+    __shared__ float lred[8];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int row0 = (blockIdx.x * 8 + warp) * R;
+    ttfsi_sgemm::pdl_launch();
+    ttfsi_sgemm::pdl_wait();
+    float sum[R], shift[R], gmean[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) sum[r] = 0.f;
+    for (int k = lane; k < a.n_out; k += 32) {
+        const float b = a.bias[k];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            if (row0 + r >= a.B) break;
+            float *y = a.Y + (long long)(row0 + r) * a.ldy + k;
+            float v = 0.f;
+            for (int z = 0; z < a.slices; ++z) v += y[z * a.zstride];
+            v += b;
+            *y = v;
+            if (k > 0) sum[r] += v;
         }
-        __threadfence();
     }
-    __syncthreads();
-    if (threadIdx.x == 0 && threadIdx.y == 0)
-        s_last = atomicAdd(arrivals + blockIdx.x, 1) == (int)gridDim.y - 1;
-    __syncthreads();
-    if (!s_last) return;
-    if (threadIdx.y == 0) {
-        __threadfence();
-        if (c < N) {
-            float t = 0.f;
-            for (int k = 0; k < (int)gridDim.y; ++k) t += __ldcg(part + (long long)k * N + c);
-            out[c] = t;
+    float loss = 0.f;
+    const float scale = 2.0f / ((float)a.B * (float)a.n_out);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const bool in = row0 + r < a.B;
+        shift[r] = in ? (a.target[row0 + r] - warp_sum(sum[r])) / (float)(a.n_out - 1) : 0.f;
+        gmean[r] = 0.f;
+    }
+    for (int k = lane; k < a.n_out; k += 32) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            if (row0 + r >= a.B) break;
+            const float p = (k == 0) ? a.v_empty : a.Y[(long long)(row0 + r) * a.ldy + k] + shift[r];
+            const long long at = (long long)(row0 + r) * a.n_out + k;
+            if (a.phi) a.phi[at] = p;
+            if (a.labels) {
+                const float e = p - a.labels[at];
+                loss += e * e;
+                if (k > 0) gmean[r] += scale * e;
+            }
         }
-        if (threadIdx.x == 0) arrivals[blockIdx.x] = 0;
     }
-}
-
-// Sum of the per-instance losses, one block, fixed order.
-__global__ void sum_kernel(const float *x, int n, float scale, float *out) {
-    __shared__ float red[256];
-    float s = 0.f;
-    for (int i = threadIdx.x; i < n; i += 256) s += x[i];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+    if (!a.labels) return;
+#pragma unroll
+    for (int r = 0; r < R; ++r) gmean[r] = warp_sum(gmean[r]) / (float)(a.n_out - 1);
+    loss = warp_sum(loss);
+    if (lane == 0) lred[warp] = loss;
+    for (int k0 = 0; k0 < a.ld_dyb; k0 += 32) {
+        const int k = k0 + lane;
+        float col = 0.f;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            if (row0 + r >= a.B) break;
+            float g = 0.f;
+            if (k > 0 && k < a.n_out) {
+                const float p = a.Y[(long long)(row0 + r) * a.ldy + k] + shift[r];
+                g = scale * (p - a.labels[(long long)(row0 + r) * a.n_out + k]) - gmean[r];
+            }
+            if (k < a.ld_dyb) a.dYb[(long long)(row0 + r) * a.ld_dyb + k] = __float2bfloat16_rn(g);
+            col += g;
+        }
+        red[warp][lane] = col;
+        __syncthreads();
+        if (warp == 0 && k < a.n_out) {
+            float t = 0.f;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) t += red[w][lane];
+            a.col_part[(long long)blockIdx.x * a.n_out + k] = t;
+        }
         __syncthreads();
     }
-    if (threadIdx.x == 0) *out = red[0] * scale;
+    if (threadIdx.x == 0) {
+        float t = 0.f;
+        for (int w = 0; w < 8; ++w) t += lred[w];
+        a.loss_part[blockIdx.x] = t;
+    }
 }
 
-// Adam (Kingma & Ba): m = b1 m + (1-b1) g, v = b2 v + (1-b2) g^2,
-// p -= lr (m / (1 - b1^t)) / (sqrt(v / (1 - b2^t)) + eps), over a flat buffer.
-__global__ void adam_kernel(float *p, float *m, float *v, const float *g, long long n, float lr, float b1, float b2,
-                            float eps, float c1, float c2) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.f - b1) * gi;
-        const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+// The end of a step: every gradient is the sum of partial results in a fixed
+// order (K slices of the weight gradients, row blocks of the bias gradients),
+// and with `update` Adam (Kingma & Ba) follows on the spot, m = b1 m +
+// (1-b1) g, v = b2 v + (1-b2) g^2, p -= lr (m / (1 - b1^t)) / (sqrt(v /
+// (1 - b2^t)) + eps), with the BF16 copy of a weight that the products read.
+// Four weights per thread; a warp per 32 columns of a bias; one block more
+// adds the loss.
+struct FinishArgs {
+    float *p, *m, *v, *g;
+    const float *wpart[3];  // [slices][stride]
+    long long wstride[3];
+    int wslices[3];
+    long long woff[3], wn[3];  // multiples of 4
+    bf16 *wb[3];
+    const float *bpart[3];  // [parts][bn]
+    int bparts[3], bn[3];
+    long long boff[3];
+    const float *loss_part;
+    int loss_parts;
+    float loss_scale;
+    float *loss;  // or null
+    int bias_blocks;  // blocks of 8 warps ahead of the weights' blocks
+    int update;
+    float lr, b1, b2, eps, c1, c2;
+};
+
+__device__ __forceinline__ float adam_one(const FinishArgs &a, float g, float &m, float &v, float p) {
+    m = a.b1 * m + (1.f - a.b1) * g;
+    v = a.b2 * v + (1.f - a.b2) * g * g;
+    return p - a.lr * (m / a.c1) / (sqrtf(v / a.c2) + a.eps);
+}
+
+__global__ void __launch_bounds__(256) finish_kernel(const __grid_constant__ FinishArgs a) {
+    ttfsi_sgemm::pdl_launch();
+    ttfsi_sgemm::pdl_wait();
+    if ((int)blockIdx.x < a.bias_blocks) {
+        const int lane = threadIdx.x & 31;
+        int w = (int)blockIdx.x * 8 + (threadIdx.x >> 5);
+        if (w == 0) {
+            if (!a.loss) return;
+            float t = 0.f;
+            for (int i = lane; i < a.loss_parts; i += 32) t += a.loss_part[i];
+            t = warp_sum(t);
+            if (lane == 0) *a.loss = t * a.loss_scale;
+            return;
+        }
+        --w;
+        int k = 0;
+        while (k < 3 && w >= (a.bn[k] + 31) / 32) w -= (a.bn[k++] + 31) / 32;
+        const int c = w * 32 + lane;
+        if (k >= 3 || c >= a.bn[k]) return;
+        float g = 0.f;
+#pragma unroll 16
+        for (int i = 0; i < a.bparts[k]; ++i) g += a.bpart[k][(long long)i * a.bn[k] + c];
+        const long long at = a.boff[k] + c;
+        a.g[at] = g;
+        if (a.update) {
+            float m = a.m[at], v = a.v[at];
+            a.p[at] = adam_one(a, g, m, v, a.p[at]);
+            a.m[at] = m;
+            a.v[at] = v;
+        }
+        return;
     }
+    long long i = ((long long)(blockIdx.x - a.bias_blocks) * 256 + threadIdx.x) * 4;
+    int k = 0;
+    while (k < 3 && i >= a.wn[k]) i -= a.wn[k++];
+    if (k >= 3) return;
+    const long long at = a.woff[k] + i;
+    float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+    for (int z = 0; z < a.wslices[k]; ++z) {
+        const float4 x = *reinterpret_cast<const float4 *>(a.wpart[k] + z * a.wstride[k] + i);
+        g.x += x.x;
+        g.y += x.y;
+        g.z += x.z;
+        g.w += x.w;
+    }
+    *reinterpret_cast<float4 *>(a.g + at) = g;
+    if (!a.update) return;
+    float4 m = *reinterpret_cast<float4 *>(a.m + at), v = *reinterpret_cast<float4 *>(a.v + at);
+    float4 p = *reinterpret_cast<float4 *>(a.p + at);
+    p.x = adam_one(a, g.x, m.x, v.x, p.x);
+    p.y = adam_one(a, g.y, m.y, v.y, p.y);
+    p.z = adam_one(a, g.z, m.z, v.z, p.z);
+    p.w = adam_one(a, g.w, m.w, v.w, p.w);
+    *reinterpret_cast<float4 *>(a.m + at) = m;
+    *reinterpret_cast<float4 *>(a.v + at) = v;
+    *reinterpret_cast<float4 *>(a.p + at) = p;
+    uint2 b;
+    b.x = ttfsi_sgemm::pack_bf16(p.x, p.y);
+    b.y = ttfsi_sgemm::pack_bf16(p.z, p.w);
+    *reinterpret_cast<uint2 *>(a.wb[k] + i) = b;
 }
 
 // Surrogate residual of each instance on its sampled coalitions:
@@ -339,21 +376,24 @@ int grid_for(long long n) {
 }  // namespace ttfsi_student
 
 struct tt_fsi_student_s {
-    int d = 0, H = 0, n_out = 0, n_pad = 0, max_batch = 0, ldB = 0;
+    int d = 0, H = 0, n_out = 0, n_pad = 0, max_batch = 0, ldy = 0;
     long long n_params = 0;
     long long off_W1 = 0, off_b1 = 0, off_W2 = 0, off_b2 = 0, off_W3 = 0, off_b3 = 0;
     float *params = nullptr, *m = nullptr, *v = nullptr, *grads = nullptr;
-    __nv_bfloat16 *W1b = nullptr, *W2b = nullptr, *W2bT = nullptr, *W3b = nullptr, *W3bT = nullptr;
-    __nv_bfloat16 *Xb = nullptr, *XbT = nullptr, *A1 = nullptr, *A1T = nullptr, *A2 = nullptr, *A2T = nullptr;
-    __nv_bfloat16 *dYb = nullptr, *dYt = nullptr, *dH2 = nullptr, *dH2T = nullptr, *dH1T = nullptr;
-    float *Z1 = nullptr, *Z2 = nullptr, *Y = nullptr, *dYf = nullptr, *dH2f = nullptr, *dH1f = nullptr;
-    float *loss_rows = nullptr;
-    float *colpart = nullptr;  // column-sum partials [ceil(max_batch / 256)][max(H, n_out)]
-    int *colarrive = nullptr;  // column-sum arrival counters [ceil(max(H, n_out) / 32)], zero between calls
-    float *gpart = nullptr;    // K-slice partial products of the weight gradients
+    __nv_bfloat16 *W1b = nullptr, *W2b = nullptr, *W3b = nullptr;
+    __nv_bfloat16 *Xb = nullptr, *A1 = nullptr, *A2 = nullptr, *dYb = nullptr, *dH2 = nullptr, *dH1 = nullptr;
+    float *Z1 = nullptr, *Z2 = nullptr;
+    float *Y = nullptr;                                            // K slices of the output layer
+    float *part1 = nullptr, *part2 = nullptr, *part3 = nullptr;    // K slices of the weight gradients
+    float *col1 = nullptr, *col2 = nullptr, *col3 = nullptr;       // row-block sums of the bias gradients
+    float *loss_part = nullptr;
     int *err = nullptr;
     float lr = 1e-3f, beta1 = 0.9f, beta2 = 0.999f, eps = 1e-8f;
     long long step = 0;
+    // the products of a batch of plan_B instances (their tensor maps name the
+    // handle's own buffers and the batch's row count)
+    int plan_B = 0;
+    ttfsi_sgemm::Jobs f1_train, f1, f2_train, f2, f3, b3, b2, b1;
     std::vector<void *> allocs;
 };
 
@@ -371,142 +411,242 @@ cudaError_t st_alloc(tt_fsi_student_s *s, T **p, size_t count) {
     return e;
 }
 
-tt_fsi_status gemm(const bf16 *A, int lda, const bf16 *B, int ldb, int M, int N, int K, const float *bias, int act,
-                   const float *dz, int ldz, float *Cf, int ldcf, bf16 *Cb, int ldcb, bf16 *Ct, int ldct, int *err,
-                   cudaStream_t st, float *gpart = nullptr) {
-    ttfsi_gemm::GemmArgs a{};
-    a.A = A;
-    a.B = B;
-    a.lda = lda;
-    a.ldb = ldb;
-    a.M = M;
-    a.N = N;
-    a.K = K;
-    a.bias = bias;
-    a.act = act;
-    a.dgelu_z = dz;
-    a.ldz = ldz;
-    a.Cf = Cf;
-    a.ldcf = ldcf;
-    a.Cb = Cb;
-    a.ldcb = ldcb;
-    a.Ct = Ct;
-    a.ldct = ldct;
-    a.err = err;
-    // plain products with a long K (the weight gradients) are split over K
-    // into the student's partial buffer and summed in slice order
-    const int kbc = (!act && !dz && !Cb && !Ct && Cf && gpart) ? split_kbc(M, N, K) : 0;
-    if (kbc > 0) {
-        const int nk = (K + ttfsi_gemm::BK - 1) / ttfsi_gemm::BK, slices = (nk + kbc - 1) / kbc;
-        a.kbc = kbc;
-        a.bias = nullptr;  // added once, in the slice sum
-        a.Cf = gpart;
-        a.cf_zstride = (long long)M * ldcf;
-        tt_fsi_status r = gemm_launch(a, st);
-        if (r != TT_FSI_OK) return r;
-        const long long n = (long long)M * N;
-        ksum_kernel<<<(unsigned)std::min<long long>((n + 255) / 256, 4096), 256, 0, st>>>(gpart, a.cf_zstride, slices, M,
-                                                                                          N, ldcf, bias, Cf);
-        return st_status(cudaGetLastError());
-    }
-    return gemm_launch(a, st);
+// Launches a kernel of the step as the programmatic dependent of the one
+// before it: its CTAs are placed and set up while that one drains, and every
+// kernel of the chain waits for the full completion of its predecessor
+// (griddepcontrol.wait) before it reads or writes memory.
+template <typename... P, typename... A>
+tt_fsi_status chain(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st, A &&...args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return st_status(cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...));
 }
 
-void to_bf16(const float *W, int rows, int cols, int rows_pad, bf16 *Wb, bf16 *Wt, int ldt, cudaStream_t st) {
-    const dim3 grid((unsigned)((cols + 31) / 32), (unsigned)((rows_pad + 31) / 32));
-    ttfsi_student::to_bf16_tiled_kernel<<<grid, dim3(32, 8), 0, st>>>(W, rows, cols, rows_pad, Wb, Wt, ldt);
+bool encode_map(CUtensorMap *map, CUtensorMapDataType type, int elem, const void *ptr, long long rows, int cols, int ld,
+                int box_cols, int box_rows) {
+    PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
+    if (!encode) return false;
+    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)ld * elem};
+    const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
+    const cuuint32_t estr[2] = {1, 1};
+    return encode(map, type, 2, const_cast<void *>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Bias gradient: column sums of an FP32 [M, N] matrix (fixed order).
-void colsum(tt_fsi_student_s *s, const float *X, int M, int N, float *out, cudaStream_t st) {
-    const int slabs = (M + 255) / 256;
-    ttfsi_student::colsum_kernel<<<dim3((unsigned)((N + 31) / 32), (unsigned)slabs), dim3(32, 8), 0, st>>>(
-        X, M, N, s->colpart, s->colarrive, out);
+// K slices of a product: enough for two tiles per SM, at least 4 K blocks each.
+void k_split(int M, int N, int K, int &kbc, int &slices) {
+    using namespace ttfsi_gemm;
+    const int tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN), nk = (K + BK - 1) / BK;
+    slices = std::max(1, std::min((2 * 152 + tiles - 1) / tiles, nk / 4));
+    kbc = (nk + slices - 1) / slices;
+    slices = (nk + kbc - 1) / kbc;
 }
 
-// BF16 copies of the three weight matrices (and the transposes the backward
-// pass reads), one launch.
-tt_fsi_status refresh_bf16(tt_fsi_student_s *s, cudaStream_t st) {
-    using ttfsi_student::CastJob;
-    ttfsi_student::CastJobs jobs{};
-    auto add = [&](const float *W, int rows, int cols, int rows_pad, bf16 *Wb, bf16 *Wt, int ldt) {
-        CastJob &c = jobs.j[jobs.n];
-        c.W = W;
-        c.Wb = Wb;
-        c.Wt = Wt;
-        c.rows = rows;
-        c.cols = cols;
-        c.rows_pad = rows_pad;
-        c.ldt = ldt;
-        c.tiles_x = (cols + 31) / 32;
-        c.first = jobs.n ? jobs.j[jobs.n - 1].first + jobs.j[jobs.n - 1].tiles_x * ((jobs.j[jobs.n - 1].rows_pad + 31) / 32)
-                         : 0;
-        ++jobs.n;
-    };
-    add(s->params + s->off_W1, s->H, s->d, s->H, s->W1b, nullptr, 0);
-    add(s->params + s->off_W2, s->H, s->H, s->H, s->W2b, s->W2bT, s->H);
-    add(s->params + s->off_W3, s->n_out, s->H, s->n_pad, s->W3b, s->W3bT, s->n_pad);
-    const CastJob &last = jobs.j[jobs.n - 1];
-    const unsigned blocks = (unsigned)(last.first + last.tiles_x * ((last.rows_pad + 31) / 32));
-    ttfsi_student::to_bf16_multi_kernel<<<blocks, dim3(32, 8), 0, st>>>(jobs);
-    return st_status(cudaGetLastError());
+int round_up(int n, int to) { return (n + to - 1) / to * to; }
+
+// A product of the step.  op = 1: the operand is stored [K, rows].
+bool make_job(ttfsi_sgemm::Job &j, const bf16 *A, int lda, int a_mn, const bf16 *B, int ldb, int b_mn, int M, int N,
+              int K, bool split) {
+    using namespace ttfsi_gemm;
+    const auto T = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+    j.M = M;
+    j.N = N;
+    j.K = K;
+    j.a_mn = a_mn;
+    j.b_mn = b_mn;
+    j.tiles_m = (M + BM - 1) / BM;
+    j.tiles_n = (N + BN - 1) / BN;
+    int slices = 1;
+    j.kbc = (K + BK - 1) / BK;
+    if (split) k_split(M, N, K, j.kbc, slices);
+    j.zrows = round_up(M, 32);
+    j.blocks = j.tiles_m * j.tiles_n * slices;
+    return (a_mn ? encode_map(&j.A, T, 2, A, K, M, lda, 64, BK) : encode_map(&j.A, T, 2, A, M, K, lda, BK, BM)) &&
+           (b_mn ? encode_map(&j.B, T, 2, B, K, N, ldb, 64, BK) : encode_map(&j.B, T, 2, B, N, K, ldb, BK, BN));
 }
 
-// Forward pass into s->Y (raw outputs); `train` also keeps what the backward
-// pass needs (transposed activations).
-tt_fsi_status forward(tt_fsi_student_s *s, const float *x, int B, bool train, cudaStream_t st) {
-    using namespace ttfsi_student;
-    to_bf16(x, B, s->d, B, s->Xb, train ? s->XbT : nullptr, s->ldB, st);
-    tt_fsi_status r = st_status(cudaGetLastError());
-    if (r != TT_FSI_OK) return r;
+int job_slices(const ttfsi_sgemm::Job &j) { return j.blocks / (j.tiles_m * j.tiles_n); }
+
+bool out_partial(ttfsi_sgemm::Job &j, float *F, int ld) {
+    j.kind = ttfsi_sgemm::kPartial;
+    return encode_map(&j.F, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, F, (long long)j.zrows * job_slices(j), j.N, ld, 32, 32);
+}
+
+bool out_act(ttfsi_sgemm::Job &j, const float *bias, float *Z, bf16 *Hb) {
+    j.kind = ttfsi_sgemm::kAct;
+    j.bias = bias;
+    j.has_f = Z != nullptr;
+    return (!Z || encode_map(&j.F, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, Z, j.M, j.N, j.N, 32, 32)) &&
+           encode_map(&j.Hb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Hb, j.M, j.N, j.N, 64, 32);
+}
+
+bool out_dgelu(ttfsi_sgemm::Job &j, const float *Z, bf16 *Hb, float *colpart) {
+    j.kind = ttfsi_sgemm::kDgelu;
+    j.colpart = colpart;
+    return encode_map(&j.Z, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, Z, j.M, j.N, j.N, 32, 32) &&
+           encode_map(&j.Hb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Hb, j.M, j.N, j.N, 64, 32);
+}
+
+// The products for batches of B instances; made again when B changes.
+tt_fsi_status plan_batch(tt_fsi_student_s *s, int B) {
+    if (s->plan_B == B) return TT_FSI_OK;
+    s->plan_B = 0;
+    const int d = s->d, H = s->H, n_out = s->n_out, n_pad = s->n_pad;
     const float *P = s->params;
-    // the FP32 pre-activations Z1, Z2 and the transposed activations are
-    // read only by the backward pass
-    r = gemm(s->Xb, s->d, s->W1b, s->d, B, s->H, s->d, P + s->off_b1, 1, nullptr, 0, train ? s->Z1 : nullptr, s->H,
-             s->A1, s->H, train ? s->A1T : nullptr, s->ldB, s->err, st);
-    if (r != TT_FSI_OK) return r;
-    r = gemm(s->A1, s->H, s->W2b, s->H, B, s->H, s->H, P + s->off_b2, 1, nullptr, 0, train ? s->Z2 : nullptr, s->H,
-             s->A2, s->H, train ? s->A2T : nullptr, s->ldB, s->err, st);
-    if (r != TT_FSI_OK) return r;
-    return gemm(s->A2, s->H, s->W3b, s->H, B, s->n_out, s->H, P + s->off_b3, 0, nullptr, 0, s->Y, s->n_out, nullptr, 0,
-                nullptr, 0, s->err, st, s->gpart);
+    bool ok = true;
+    for (auto *j : {&s->f1_train, &s->f1, &s->f2_train, &s->f2, &s->f3, &s->b3, &s->b2, &s->b1}) {
+        memset(j, 0, sizeof(*j));
+        j->err = s->err;
+    }
+    for (auto *j : {&s->f1_train, &s->f1})
+        ok = ok && make_job(j->j[0], s->Xb, d, 0, s->W1b, d, 0, B, H, d, false) &&
+             out_act(j->j[0], P + s->off_b1, j == &s->f1_train ? s->Z1 : nullptr, s->A1);
+    for (auto *j : {&s->f2_train, &s->f2})
+        ok = ok && make_job(j->j[0], s->A1, H, 0, s->W2b, H, 0, B, H, H, false) &&
+             out_act(j->j[0], P + s->off_b2, j == &s->f2_train ? s->Z2 : nullptr, s->A2);
+    ok = ok && make_job(s->f3.j[0], s->A2, H, 0, s->W3b, H, 0, B, n_out, H, true) &&
+         out_partial(s->f3.j[0], s->Y, s->ldy);
+    // dH2 = (dY W3) gelu'(Z2) and dW3 = dY^T A2
+    ok = ok && make_job(s->b3.j[0], s->dYb, n_pad, 0, s->W3b, H, 1, B, H, n_out, false) &&
+         out_dgelu(s->b3.j[0], s->Z2, s->dH2, s->col2) &&
+         make_job(s->b3.j[1], s->dYb, n_pad, 1, s->A2, H, 1, n_out, H, B, true) &&
+         out_partial(s->b3.j[1], s->part3, H);
+    // dW2 = dH2^T A1 and dH1 = (dH2 W2) gelu'(Z1)
+    ok = ok && make_job(s->b2.j[0], s->dH2, H, 1, s->A1, H, 1, H, H, B, true) &&
+         out_partial(s->b2.j[0], s->part2, H) &&
+         make_job(s->b2.j[1], s->dH2, H, 0, s->W2b, H, 1, B, H, H, false) &&
+         out_dgelu(s->b2.j[1], s->Z1, s->dH1, s->col1);
+    // dW1 = dH1^T X
+    ok = ok && make_job(s->b1.j[0], s->dH1, H, 1, s->Xb, d, 1, H, d, B, true) && out_partial(s->b1.j[0], s->part1, d);
+    if (!ok) return TT_FSI_ERR_CUDA;
+    s->plan_B = B;
+    return TT_FSI_OK;
 }
 
-// Gradients of the mean squared error of the projected outputs into s->grads.
-tt_fsi_status backward(tt_fsi_student_s *s, const float *labels, const float *target, float v_empty, int B,
-                       float *loss_dev, cudaStream_t st) {
-    using namespace ttfsi_student;
-    const int warps_per_block = 8;
-    project_loss_kernel<<<(B + warps_per_block - 1) / warps_per_block, 32 * warps_per_block, 0, st>>>(
-        s->Y, B, s->n_out, target, v_empty, nullptr, labels, s->loss_rows, s->dYf, s->dYb, s->n_pad, nullptr, 0);
-    // dY^T (rows n_out..n_pad of dYt stay zero)
-    to_bf16(s->dYf, B, s->n_out, B, nullptr, s->dYt, s->ldB, st);
-    tt_fsi_status r = st_status(cudaGetLastError());
+tt_fsi_status run_jobs(const ttfsi_sgemm::Jobs &j, cudaStream_t st) {
+    return chain(ttfsi_sgemm::student_gemm_kernel, (unsigned)(j.j[0].blocks + j.j[1].blocks), ttfsi_sgemm::SG_THREADS,
+                 ttfsi_sgemm::SG_SMEM, st, j);
+}
+
+// BF16 copies of the three weight matrices (a step keeps them up to date itself).
+tt_fsi_status refresh_bf16(tt_fsi_student_s *s, cudaStream_t st) {
+    ttfsi_student::CastJobs c{};
+    const long long H = s->H;
+    c.src[0] = s->params + s->off_W1;
+    c.dst[0] = s->W1b;
+    c.n[0] = H * s->d;
+    c.src[1] = s->params + s->off_W2;
+    c.dst[1] = s->W2b;
+    c.n[1] = H * H;
+    c.src[2] = s->params + s->off_W3;
+    c.dst[2] = s->W3b;
+    c.n[2] = H * s->n_out;
+    return chain(ttfsi_student::to_bf16_kernel, (unsigned)ttfsi_student::grid_for(c.n[0] + c.n[1] + c.n[2]), 256, 0, st,
+                 c);
+}
+
+// Forward pass up to the K slices of the raw outputs; `train` also keeps the
+// FP32 pre-activations, which only the backward pass reads.
+tt_fsi_status forward(tt_fsi_student_s *s, const float *x, int B, bool train, cudaStream_t st) {
+    tt_fsi_status r = plan_batch(s, B);
     if (r != TT_FSI_OK) return r;
-    if (loss_dev) sum_kernel<<<1, 256, 0, st>>>(s->loss_rows, B, 1.0f / ((float)B * s->n_out), loss_dev);
-    float *G = s->grads;
-    // layer 3
-    r = gemm(s->dYt, s->ldB, s->A2T, s->ldB, s->n_out, s->H, B, nullptr, 0, nullptr, 0, G + s->off_W3, s->H, nullptr, 0,
-             nullptr, 0, s->err, st, s->gpart);
+    ttfsi_student::CastJobs c{};
+    c.src[0] = x;
+    c.dst[0] = s->Xb;
+    c.n[0] = (long long)B * s->d;
+    r = chain(ttfsi_student::to_bf16_kernel, (unsigned)ttfsi_student::grid_for(c.n[0]), 256, 0, st, c);
+    if (r == TT_FSI_OK) r = run_jobs(train ? s->f1_train : s->f1, st);
+    if (r == TT_FSI_OK) r = run_jobs(train ? s->f2_train : s->f2, st);
+    if (r == TT_FSI_OK) r = run_jobs(s->f3, st);
+    return r;
+}
+
+constexpr int kTrainRows = 4;  // rows per warp of the projection in training
+
+ttfsi_student::ProjectArgs project_args(tt_fsi_student_s *s, const float *target, float v_empty, int B) {
+    const ttfsi_sgemm::Job &j = s->f3.j[0];
+    ttfsi_student::ProjectArgs a{};
+    a.Y = s->Y;
+    a.slices = job_slices(j);
+    a.ldy = s->ldy;
+    a.zstride = (long long)j.zrows * s->ldy;
+    a.bias = s->params + s->off_b3;
+    a.B = B;
+    a.n_out = s->n_out;
+    a.target = target;
+    a.v_empty = v_empty;
+    return a;
+}
+
+// Forward, backward and the gradients (with `update`, Adam too).
+tt_fsi_status step(tt_fsi_student_s *s, const float *x, const float *labels, const float *target, float v_empty, int B,
+                   float *loss_dev, bool update, cudaStream_t st) {
+    tt_fsi_status r = forward(s, x, B, true, st);
     if (r != TT_FSI_OK) return r;
-    colsum(s, s->dYf, B, s->n_out, G + s->off_b3, st);
-    r = gemm(s->dYb, s->n_pad, s->W3bT, s->n_pad, B, s->H, s->n_pad, nullptr, 0, s->Z2, s->H, s->dH2f, s->H, s->dH2,
-             s->H, s->dH2T, s->ldB, s->err, st);
+    const int pblocks = (B + 8 * kTrainRows - 1) / (8 * kTrainRows), mtiles = (B + ttfsi_gemm::BM - 1) / ttfsi_gemm::BM;
+    ttfsi_student::ProjectArgs p = project_args(s, target, v_empty, B);
+    p.labels = labels;
+    p.loss_part = s->loss_part;
+    p.col_part = s->col3;
+    p.dYb = s->dYb;
+    p.ld_dyb = s->n_pad;
+    r = chain(ttfsi_student::project_kernel<kTrainRows>, (unsigned)pblocks, 256, 0, st, p);
+    if (r == TT_FSI_OK) r = run_jobs(s->b3, st);
+    if (r == TT_FSI_OK) r = run_jobs(s->b2, st);
+    if (r == TT_FSI_OK) r = run_jobs(s->b1, st);
     if (r != TT_FSI_OK) return r;
-    // layer 2
-    colsum(s, s->dH2f, B, s->H, G + s->off_b2, st);
-    r = gemm(s->dH2T, s->ldB, s->A1T, s->ldB, s->H, s->H, B, nullptr, 0, nullptr, 0, G + s->off_W2, s->H, nullptr, 0,
-             nullptr, 0, s->err, st, s->gpart);
-    if (r != TT_FSI_OK) return r;
-    r = gemm(s->dH2, s->H, s->W2bT, s->H, B, s->H, s->H, nullptr, 0, s->Z1, s->H, s->dH1f, s->H, nullptr, 0, s->dH1T,
-             s->ldB, s->err, st);
-    if (r != TT_FSI_OK) return r;
-    // layer 1
-    colsum(s, s->dH1f, B, s->H, G + s->off_b1, st);
-    r = gemm(s->dH1T, s->ldB, s->XbT, s->ldB, s->H, s->d, B, nullptr, 0, nullptr, 0, G + s->off_W1, s->d, nullptr, 0,
-             nullptr, 0, s->err, st, s->gpart);
-    if (r != TT_FSI_OK) return r;
-    return st_status(cudaGetLastError());
+
+    ttfsi_student::FinishArgs f{};
+    f.p = s->params;
+    f.m = s->m;
+    f.v = s->v;
+    f.g = s->grads;
+    const ttfsi_sgemm::Job *jobs[3] = {&s->b1.j[0], &s->b2.j[0], &s->b3.j[1]};
+    float *parts[3] = {s->part1, s->part2, s->part3}, *cols[3] = {s->col1, s->col2, s->col3};
+    const long long woff[3] = {s->off_W1, s->off_W2, s->off_W3}, boff[3] = {s->off_b1, s->off_b2, s->off_b3};
+    bf16 *wb[3] = {s->W1b, s->W2b, s->W3b};
+    long long weights = 0;
+    int warps = 1;  // the loss
+    for (int k = 0; k < 3; ++k) {
+        f.wpart[k] = parts[k];
+        f.wstride[k] = (long long)jobs[k]->zrows * jobs[k]->N;
+        f.wslices[k] = job_slices(*jobs[k]);
+        f.woff[k] = woff[k];
+        f.wn[k] = (long long)jobs[k]->M * jobs[k]->N;
+        f.wb[k] = wb[k];
+        f.bpart[k] = cols[k];
+        f.bparts[k] = k == 2 ? pblocks : mtiles;
+        f.bn[k] = k == 2 ? s->n_out : s->H;
+        f.boff[k] = boff[k];
+        weights += f.wn[k];
+        warps += (f.bn[k] + 31) / 32;
+    }
+    f.loss_part = s->loss_part;
+    f.loss_parts = pblocks;
+    f.loss_scale = 1.0f / ((float)B * s->n_out);
+    f.loss = loss_dev;
+    f.bias_blocks = (warps + 7) / 8;
+    f.update = update;
+    if (update) {
+        s->step += 1;
+        f.lr = s->lr;
+        f.b1 = s->beta1;
+        f.b2 = s->beta2;
+        f.eps = s->eps;
+        f.c1 = 1.0f - (float)std::pow((double)s->beta1, (double)s->step);
+        f.c2 = 1.0f - (float)std::pow((double)s->beta2, (double)s->step);
+    }
+    return chain(ttfsi_student::finish_kernel, (unsigned)(f.bias_blocks + (weights / 4 + 255) / 256), 256, 0, st, f);
 }
 
 void student_free(tt_fsi_student_s *s) {
@@ -530,7 +670,7 @@ tt_fsi_status tt_fsi_student_create(int d, int hidden, int n_out, int max_batch,
     s->n_out = n_out;
     s->n_pad = (n_out + 15) / 16 * 16;
     s->max_batch = max_batch;
-    s->ldB = (max_batch + 7) / 8 * 8;
+    s->ldy = round_up(n_out, 4);  // 16-byte rows
     long long o = 0;
     s->off_W1 = o;
     o += (long long)hidden * d;
@@ -545,7 +685,7 @@ tt_fsi_status tt_fsi_student_create(int d, int hidden, int n_out, int max_batch,
     s->off_b3 = o;
     o += n_out;
     s->n_params = o;
-    const size_t Bm = (size_t)s->ldB, H = (size_t)hidden;
+    const size_t Bm = (size_t)max_batch, H = (size_t)hidden;
     cudaError_t e = cudaSuccess;
     auto A = [&](auto **p, size_t n) {
         if (e == cudaSuccess) e = st_alloc(s, p, n);
@@ -556,47 +696,50 @@ tt_fsi_status tt_fsi_student_create(int d, int hidden, int n_out, int max_batch,
     A(&s->grads, (size_t)o);
     A(&s->W1b, H * d);
     A(&s->W2b, H * H);
-    A(&s->W2bT, H * H);
     A(&s->W3b, (size_t)s->n_pad * H);
-    A(&s->W3bT, H * s->n_pad);
     A(&s->Xb, Bm * d);
-    A(&s->XbT, (size_t)d * Bm);
     A(&s->A1, Bm * H);
-    A(&s->A1T, H * Bm);
     A(&s->A2, Bm * H);
-    A(&s->A2T, H * Bm);
     A(&s->Z1, Bm * H);
     A(&s->Z2, Bm * H);
-    A(&s->Y, Bm * n_out);
-    A(&s->dYf, Bm * n_out);
     A(&s->dYb, Bm * s->n_pad);
-    A(&s->dYt, (size_t)s->n_pad * Bm);
-    A(&s->dH2f, Bm * H);
     A(&s->dH2, Bm * H);
-    A(&s->dH2T, H * Bm);
-    A(&s->dH1f, Bm * H);
-    A(&s->dH1T, H * Bm);
-    A(&s->loss_rows, Bm);
-    A(&s->colpart, ((Bm + 255) / 256) * (size_t)std::max(hidden, n_out));
-    A(&s->colarrive, ((size_t)std::max(hidden, n_out) + 31) / 32);
+    A(&s->dH1, Bm * H);
+    const size_t mtiles = (Bm + ttfsi_gemm::BM - 1) / ttfsi_gemm::BM, pblocks = (Bm + 8 * kTrainRows - 1) / (8 * kTrainRows);
+    A(&s->col1, mtiles * H);
+    A(&s->col2, mtiles * H);
+    A(&s->col3, pblocks * n_out);
+    A(&s->loss_part, pblocks);
     {
-        // the largest split product: the weight gradients W3 [n_out, H], W2 [H, H], W1 [H, d] with
-        // K = max_batch
-        size_t need = 0;
-        // (and the forward output layer [max_batch, n_out] with K = H)
-        const int shapes[4][3] = {{n_out, hidden, max_batch}, {hidden, hidden, max_batch}, {hidden, d, max_batch},
-                                  {max_batch, n_out, hidden}};
-        for (auto &sh : shapes) {
-            const int kbc = split_kbc(sh[0], sh[1], sh[2]);
-            if (!kbc) continue;
-            const int nk = (sh[2] + ttfsi_gemm::BK - 1) / ttfsi_gemm::BK;
-            need = std::max(need, (size_t)((nk + kbc - 1) / kbc) * sh[0] * sh[1]);
+        // K slices, for the batch size up to max_batch that needs most rows: a
+        // weight gradient has most slices at the largest batch, the output
+        // layer may have more of them at a smaller one
+        int kbc, slices;
+        auto rows = [&](int M, int N, int K) {
+            k_split(M, N, K, kbc, slices);
+            return (size_t)slices * round_up(M, 32);
+        };
+        size_t y = 0, w[3] = {0, 0, 0};
+        const int shape[3][2] = {{hidden, d}, {hidden, hidden}, {n_out, hidden}};
+        for (int b = max_batch; b > 0; b -= std::min(b, 64)) {
+            y = std::max(y, rows(b, n_out, hidden));
+            for (int k = 0; k < 3; ++k) w[k] = std::max(w[k], rows(shape[k][0], shape[k][1], b));
         }
-        if (need) A(&s->gpart, need);
+        for (int b = 128; b <= max_batch; b += 128) {
+            y = std::max(y, rows(b, n_out, hidden));
+            for (int k = 0; k < 3; ++k) w[k] = std::max(w[k], rows(shape[k][0], shape[k][1], b));
+        }
+        A(&s->Y, y * s->ldy);
+        A(&s->part1, w[0] * d);
+        A(&s->part2, w[1] * H);
+        A(&s->part3, w[2] * H);
     }
     A(&s->err, 1);
     if (e == cudaSuccess) e = cudaMemcpy(s->params, params_host, (size_t)o * sizeof(float), cudaMemcpyHostToDevice);
     tt_fsi_status r = st_status(e);
+    if (r == TT_FSI_OK)
+        r = st_status(cudaFuncSetAttribute(ttfsi_sgemm::student_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           ttfsi_sgemm::SG_SMEM));
     if (r == TT_FSI_OK) r = refresh_bf16(s, nullptr);
     if (r == TT_FSI_OK) r = st_status(cudaDeviceSynchronize());
     if (r != TT_FSI_OK) {
@@ -632,25 +775,15 @@ tt_fsi_status tt_fsi_student_gradients(tt_fsi_student s, const float *x_dev, con
                                        struct CUstream_st *stream) {
     if (!s || !x_dev || !labels_dev || !target_dev || B < 1 || B > s->max_batch) return TT_FSI_ERR_INVALID_ARG;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    tt_fsi_status r = forward(s, x_dev, B, true, st);
-    if (r == TT_FSI_OK) r = backward(s, labels_dev, target_dev, v_empty, B, loss_dev, st);
-    return r;
+    return step(s, x_dev, labels_dev, target_dev, v_empty, B, loss_dev, false, st);
 }
 
 tt_fsi_status tt_fsi_student_train_step(tt_fsi_student s, const float *x_dev, const float *labels_dev,
                                         const float *target_dev, float v_empty, int B, float *loss_dev,
                                         struct CUstream_st *stream) {
-    tt_fsi_status r = tt_fsi_student_gradients(s, x_dev, labels_dev, target_dev, v_empty, B, loss_dev, stream);
-    if (r != TT_FSI_OK) return r;
+    if (!s || !x_dev || !labels_dev || !target_dev || B < 1 || B > s->max_batch) return TT_FSI_ERR_INVALID_ARG;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    s->step += 1;
-    const float c1 = 1.0f - (float)std::pow((double)s->beta1, (double)s->step);
-    const float c2 = 1.0f - (float)std::pow((double)s->beta2, (double)s->step);
-    ttfsi_student::adam_kernel<<<ttfsi_student::grid_for(s->n_params), 256, 0, st>>>(
-        s->params, s->m, s->v, s->grads, s->n_params, s->lr, s->beta1, s->beta2, s->eps, c1, c2);
-    r = st_status(cudaGetLastError());
-    if (r == TT_FSI_OK) r = refresh_bf16(s, st);
-    return r;
+    return step(s, x_dev, labels_dev, target_dev, v_empty, B, loss_dev, true, st);
 }
 
 tt_fsi_status tt_fsi_student_predict(tt_fsi_student s, const float *x_dev, const float *target_dev, float v_empty,
@@ -659,9 +792,9 @@ tt_fsi_status tt_fsi_student_predict(tt_fsi_student s, const float *x_dev, const
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     tt_fsi_status r = forward(s, x_dev, B, false, st);
     if (r != TT_FSI_OK) return r;
-    ttfsi_student::project_loss_kernel<<<(B + 7) / 8, 256, 0, st>>>(s->Y, B, s->n_out, target_dev, v_empty, phi_dev,
-                                                                  nullptr, nullptr, nullptr, nullptr, 0, nullptr, 0);
-    return st_status(cudaGetLastError());
+    ttfsi_student::ProjectArgs p = project_args(s, target_dev, v_empty, B);
+    p.phi = phi_dev;
+    return chain(ttfsi_student::project_kernel<1>, (unsigned)((B + 7) / 8), 256, 0, st, p);
 }
 
 tt_fsi_status tt_fsi_student_get_state(tt_fsi_student s, float *params_host, float *adam_m_host, float *adam_v_host,
