@@ -148,8 +148,8 @@ __global__ void to_bf16_kernel(CastJobs c) {
 // raw outputs, dL/dY = P (2 (phi_p - phi) / (B n_out)), P = I - 11^T/(n_out-1)
 // on the non-empty coordinates, 0 on the empty one, as BF16 (the operand of
 // the backward products), its FP32 column sums over the block's rows (the bias
-// gradient's partial sums) and the block's loss.  A warp takes R rows, a block
-// 8 R; y is kept in the first slice's row, which only its own lanes read.
+// gradient's partial sums) and the block's loss.  A warp takes a row, a block
+// 8; y is kept in the first slice's row, which only its own lanes read.
 struct ProjectArgs {
     float *Y;  // [slices][zrows][ldy]
     int slices, ldy;
@@ -170,78 +170,77 @@ __device__ __forceinline__ float warp_sum(float s) {
     return s;
 }
 
-template <int R>
 __global__ void __launch_bounds__(256) project_kernel(const ProjectArgs a) {
-    __shared__ float red[8][32];
+    constexpr int C = 4;  // columns per lane in flight
+    __shared__ float red[8][32 * C];
     __shared__ float lred[8];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row0 = (blockIdx.x * 8 + warp) * R;
+    const int row = blockIdx.x * 8 + warp, n_out = a.n_out;
+    const bool in = row < a.B;
     ttfsi_sgemm::pdl_launch();
     ttfsi_sgemm::pdl_wait();
-    float sum[R], shift[R], gmean[R];
+    float *y = a.Y + (long long)(in ? row : 0) * a.ldy;
+    const long long at = (long long)(in ? row : 0) * n_out;
+    float sum = 0.f;
+    if (in)
+        for (int k0 = lane; k0 < n_out; k0 += 32 * C) {
+            float v[C] = {};
+#pragma unroll 4
+            for (int z = 0; z < a.slices; ++z)
 #pragma unroll
-    for (int r = 0; r < R; ++r) sum[r] = 0.f;
-    for (int k = lane; k < a.n_out; k += 32) {
-        const float b = a.bias[k];
+                for (int c = 0; c < C; ++c) v[c] += y[z * a.zstride + min(k0 + 32 * c, n_out - 1)];
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            if (row0 + r >= a.B) break;
-            float *y = a.Y + (long long)(row0 + r) * a.ldy + k;
-            float v = 0.f;
-            for (int z = 0; z < a.slices; ++z) v += y[z * a.zstride];
-            v += b;
-            *y = v;
-            if (k > 0) sum[r] += v;
-        }
-    }
-    float loss = 0.f;
-    const float scale = 2.0f / ((float)a.B * (float)a.n_out);
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const bool in = row0 + r < a.B;
-        shift[r] = in ? (a.target[row0 + r] - warp_sum(sum[r])) / (float)(a.n_out - 1) : 0.f;
-        gmean[r] = 0.f;
-    }
-    for (int k = lane; k < a.n_out; k += 32) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            if (row0 + r >= a.B) break;
-            const float p = (k == 0) ? a.v_empty : a.Y[(long long)(row0 + r) * a.ldy + k] + shift[r];
-            const long long at = (long long)(row0 + r) * a.n_out + k;
-            if (a.phi) a.phi[at] = p;
-            if (a.labels) {
-                const float e = p - a.labels[at];
-                loss += e * e;
-                if (k > 0) gmean[r] += scale * e;
+            for (int c = 0; c < C; ++c) {
+                const int k = k0 + 32 * c;
+                if (k >= n_out) break;
+                v[c] += a.bias[k];
+                if (k > 0) sum += v[c];
+                y[k] = v[c];
             }
         }
-    }
-    if (!a.labels) return;
+    const float shift = in ? (a.target[row] - warp_sum(sum)) / (float)(n_out - 1) : 0.f;
+    const float scale = 2.0f / ((float)a.B * (float)n_out);
+    float loss = 0.f, gsum = 0.f;
+    if (in)
+        for (int k0 = lane; k0 < n_out; k0 += 32 * C) {
+            float p[C], l[C];
 #pragma unroll
-    for (int r = 0; r < R; ++r) gmean[r] = warp_sum(gmean[r]) / (float)(a.n_out - 1);
+            for (int c = 0; c < C; ++c) {
+                const int k = min(k0 + 32 * c, n_out - 1);
+                p[c] = y[k];
+                l[c] = a.labels ? a.labels[at + k] : 0.f;
+            }
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const int k = k0 + 32 * c;
+                if (k >= n_out) break;
+                p[c] = (k == 0) ? a.v_empty : p[c] + shift;
+                if (a.phi) a.phi[at + k] = p[c];
+                const float e = p[c] - l[c];
+                loss += e * e;
+                if (k > 0) gsum += scale * e;
+            }
+        }
+    if (!a.labels) return;
+    const float gmean = warp_sum(gsum) / (float)(n_out - 1);
     loss = warp_sum(loss);
     if (lane == 0) lred[warp] = loss;
-    for (int k0 = 0; k0 < a.ld_dyb; k0 += 32) {
-        const int k = k0 + lane;
-        float col = 0.f;
+    for (int k1 = 0; k1 < a.ld_dyb; k1 += 32 * C) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            if (row0 + r >= a.B) break;
+        for (int c = 0; c < C; ++c) {
+            const int k = k1 + 32 * c + lane;
             float g = 0.f;
-            if (k > 0 && k < a.n_out) {
-                const float p = a.Y[(long long)(row0 + r) * a.ldy + k] + shift[r];
-                g = scale * (p - a.labels[(long long)(row0 + r) * a.n_out + k]) - gmean[r];
-            }
-            if (k < a.ld_dyb) a.dYb[(long long)(row0 + r) * a.ld_dyb + k] = __float2bfloat16_rn(g);
-            col += g;
+            if (in && k > 0 && k < n_out) g = scale * (y[k] + shift - a.labels[at + k]) - gmean;
+            if (in && k < a.ld_dyb) a.dYb[(long long)row * a.ld_dyb + k] = __float2bfloat16_rn(g);
+            red[warp][32 * c + lane] = g;
         }
-        red[warp][lane] = col;
         __syncthreads();
-        if (warp == 0 && k < a.n_out) {
+        const int k = k1 + (int)threadIdx.x;
+        if ((int)threadIdx.x < 32 * C && k < n_out) {
             float t = 0.f;
 #pragma unroll
-            for (int w = 0; w < 8; ++w) t += red[w][lane];
-            a.col_part[(long long)blockIdx.x * a.n_out + k] = t;
+            for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
+            a.col_part[(long long)blockIdx.x * n_out + k] = t;
         }
         __syncthreads();
     }
@@ -257,8 +256,8 @@ __global__ void __launch_bounds__(256) project_kernel(const ProjectArgs a) {
 // and with `update` Adam (Kingma & Ba) follows on the spot, m = b1 m +
 // (1-b1) g, v = b2 v + (1-b2) g^2, p -= lr (m / (1 - b1^t)) / (sqrt(v /
 // (1 - b2^t)) + eps), with the BF16 copy of a weight that the products read.
-// Four weights per thread; a warp per 32 columns of a bias; one block more
-// adds the loss.
+// Four weights per thread; a block per 32 columns of a bias, its warps over
+// the row blocks; the first block adds the loss.
 struct FinishArgs {
     float *p, *m, *v, *g;
     const float *wpart[3];  // [slices][stride]
@@ -273,7 +272,7 @@ struct FinishArgs {
     int loss_parts;
     float loss_scale;
     float *loss;  // or null
-    int bias_blocks;  // blocks of 8 warps ahead of the weights' blocks
+    int bias_blocks;  // the loss's and the biases' blocks, ahead of the weights'
     int update;
     float lr, b1, b2, eps, c1, c2;
 };
@@ -285,27 +284,34 @@ __device__ __forceinline__ float adam_one(const FinishArgs &a, float g, float &m
 }
 
 __global__ void __launch_bounds__(256) finish_kernel(const __grid_constant__ FinishArgs a) {
+    __shared__ float red[8][32];
     ttfsi_sgemm::pdl_launch();
     ttfsi_sgemm::pdl_wait();
     if ((int)blockIdx.x < a.bias_blocks) {
         const int lane = threadIdx.x & 31;
-        int w = (int)blockIdx.x * 8 + (threadIdx.x >> 5);
-        if (w == 0) {
-            if (!a.loss) return;
-            float t = 0.f;
-            for (int i = lane; i < a.loss_parts; i += 32) t += a.loss_part[i];
-            t = warp_sum(t);
-            if (lane == 0) *a.loss = t * a.loss_scale;
+        const int warp = threadIdx.x >> 5;
+        int w = (int)blockIdx.x - 1, k = 0;
+        while (w >= 0 && k < 3 && w >= (a.bn[k] + 31) / 32) w -= (a.bn[k++] + 31) / 32;
+        const int c = w * 32 + lane;
+        float g = 0.f;
+        if (w < 0) {  // the loss
+            for (int i = threadIdx.x; i < a.loss_parts; i += 256) g += a.loss_part[i];
+            g = warp_sum(g);
+        } else if (c < a.bn[k]) {
+#pragma unroll 8
+            for (int i = warp; i < a.bparts[k]; i += 8) g += a.bpart[k][(long long)i * a.bn[k] + c];
+        }
+        red[warp][lane] = g;
+        __syncthreads();
+        if (warp > 0) return;
+        g = 0.f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) g += red[i][lane];
+        if (w < 0) {
+            if (lane == 0 && a.loss) *a.loss = g * a.loss_scale;
             return;
         }
-        --w;
-        int k = 0;
-        while (k < 3 && w >= (a.bn[k] + 31) / 32) w -= (a.bn[k++] + 31) / 32;
-        const int c = w * 32 + lane;
-        if (k >= 3 || c >= a.bn[k]) return;
-        float g = 0.f;
-#pragma unroll 16
-        for (int i = 0; i < a.bparts[k]; ++i) g += a.bpart[k][(long long)i * a.bn[k] + c];
+        if (c >= a.bn[k]) return;
         const long long at = a.boff[k] + c;
         a.g[at] = g;
         if (a.update) {
@@ -349,19 +355,51 @@ __global__ void __launch_bounds__(256) finish_kernel(const __grid_constant__ Fin
 
 // Surrogate residual of each instance on its sampled coalitions:
 // g(T) = sum over scores S subset of T of phi(S);
-// r = sqrt(mean_k (g(T_k) - v(T_k))^2).  One warp per instance.
-__global__ void residual_kernel(const float *phi, int B, int n_out, const unsigned *masks, const unsigned *coal,
-                                const float *vcoal, int K, float *resid) {
+// r = sqrt(mean_k (g(T_k) - v(T_k))^2).  One warp per instance; a lane sums
+// two coalitions at a time, so that a score and its mask, the same for all
+// lanes, are read once for 64 of them, eight scores in flight (one coalition
+// and one score at a time: 15.9 us for 4096 instances, 64 coalitions, 137
+// scores).
+__global__ void __launch_bounds__(256) residual_kernel(const float *phi, int B, int n_out, const unsigned *masks,
+                                                       const unsigned *coal, const float *vcoal, int K, float *resid) {
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (warp >= B) return;
+    const float *p = phi + (long long)warp * n_out;
+    const unsigned *T = coal + (long long)warp * K;
+    const float *v = vcoal + (long long)warp * K;
     float acc = 0.f;
-    for (int k = lane; k < K; k += 32) {
-        const unsigned T = coal[(long long)warp * K + k];
-        float g = 0.f;
-        for (int q = 0; q < n_out; ++q)
-            if ((masks[q] & T) == masks[q]) g += phi[(long long)warp * n_out + q];
-        const float e = g - vcoal[(long long)warp * K + k];
-        acc += e * e;
+    for (int k = lane; k < K; k += 64) {
+        const bool two = k + 32 < K;
+        const unsigned out0 = ~T[k], out1 = two ? ~T[k + 32] : 0u;
+        const float v0 = v[k], v1 = two ? v[k + 32] : 0.f;
+        float g0 = 0.f, g1 = 0.f;
+        int q = 0;
+        for (; q + 8 <= n_out; q += 8) {
+            unsigned m[8];
+            float f[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                m[i] = __ldg(masks + q + i);
+                f[i] = __ldg(p + q + i);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                if (!(m[i] & out0)) g0 += f[i];
+                if (!(m[i] & out1)) g1 += f[i];
+            }
+        }
+        for (; q < n_out; ++q) {
+            const unsigned m = __ldg(masks + q);
+            const float f = __ldg(p + q);
+            if (!(m & out0)) g0 += f;
+            if (!(m & out1)) g1 += f;
+        }
+        const float e0 = g0 - v0;
+        acc += e0 * e0;
+        if (two) {
+            const float e1 = g1 - v1;
+            acc += e1 * e1;
+        }
     }
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (lane == 0) resid[warp] = sqrtf(acc / (float)K);
@@ -443,11 +481,14 @@ bool encode_map(CUtensorMap *map, CUtensorMapDataType type, int elem, const void
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// K slices of a product: enough for two tiles per SM, at least 4 K blocks each.
+// K slices of a product: enough for one tile per SM, at least 4 K blocks each.
+// (A step of 4096 x 1024 with slices for two tiles per SM, one, and 128 tiles:
+// 115, 102 and 106 us; the partial sums of more slices cost more than they
+// overlap.)
 void k_split(int M, int N, int K, int &kbc, int &slices) {
     using namespace ttfsi_gemm;
     const int tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN), nk = (K + BK - 1) / BK;
-    slices = std::max(1, std::min((2 * 152 + tiles - 1) / tiles, nk / 4));
+    slices = std::max(1, std::min((ttfsi_sgemm::SG_SMS + tiles - 1) / tiles, nk / 4));
     kbc = (nk + slices - 1) / slices;
     slices = (nk + kbc - 1) / kbc;
 }
@@ -529,13 +570,15 @@ tt_fsi_status plan_batch(tt_fsi_student_s *s, int B) {
     // dW1 = dH1^T X
     ok = ok && make_job(s->b1.j[0], s->dH1, H, 1, s->Xb, d, 1, H, d, B, true) && out_partial(s->b1.j[0], s->part1, d);
     if (!ok) return TT_FSI_ERR_CUDA;
+    for (auto *j : {&s->f1_train, &s->f1, &s->f2_train, &s->f2, &s->f3, &s->b3, &s->b2, &s->b1})
+        j->stages = ttfsi_sgemm::sg_stages(j->j[0].blocks + j->j[1].blocks);
     s->plan_B = B;
     return TT_FSI_OK;
 }
 
 tt_fsi_status run_jobs(const ttfsi_sgemm::Jobs &j, cudaStream_t st) {
     return chain(ttfsi_sgemm::student_gemm_kernel, (unsigned)(j.j[0].blocks + j.j[1].blocks), ttfsi_sgemm::SG_THREADS,
-                 ttfsi_sgemm::SG_SMEM, st, j);
+                 (size_t)ttfsi_sgemm::sg_smem(j.stages), st, j);
 }
 
 // BF16 copies of the three weight matrices (a step keeps them up to date itself).
@@ -571,7 +614,7 @@ tt_fsi_status forward(tt_fsi_student_s *s, const float *x, int B, bool train, cu
     return r;
 }
 
-constexpr int kTrainRows = 4;  // rows per warp of the projection in training
+constexpr int kProjectRows = 8;  // rows per block of the projection
 
 ttfsi_student::ProjectArgs project_args(tt_fsi_student_s *s, const float *target, float v_empty, int B) {
     const ttfsi_sgemm::Job &j = s->f3.j[0];
@@ -593,14 +636,14 @@ tt_fsi_status step(tt_fsi_student_s *s, const float *x, const float *labels, con
                    float *loss_dev, bool update, cudaStream_t st) {
     tt_fsi_status r = forward(s, x, B, true, st);
     if (r != TT_FSI_OK) return r;
-    const int pblocks = (B + 8 * kTrainRows - 1) / (8 * kTrainRows), mtiles = (B + ttfsi_gemm::BM - 1) / ttfsi_gemm::BM;
+    const int pblocks = (B + kProjectRows - 1) / kProjectRows, mtiles = (B + ttfsi_gemm::BM - 1) / ttfsi_gemm::BM;
     ttfsi_student::ProjectArgs p = project_args(s, target, v_empty, B);
     p.labels = labels;
     p.loss_part = s->loss_part;
     p.col_part = s->col3;
     p.dYb = s->dYb;
     p.ld_dyb = s->n_pad;
-    r = chain(ttfsi_student::project_kernel<kTrainRows>, (unsigned)pblocks, 256, 0, st, p);
+    r = chain(ttfsi_student::project_kernel, (unsigned)pblocks, 256, 0, st, p);
     if (r == TT_FSI_OK) r = run_jobs(s->b3, st);
     if (r == TT_FSI_OK) r = run_jobs(s->b2, st);
     if (r == TT_FSI_OK) r = run_jobs(s->b1, st);
@@ -616,7 +659,7 @@ tt_fsi_status step(tt_fsi_student_s *s, const float *x, const float *labels, con
     const long long woff[3] = {s->off_W1, s->off_W2, s->off_W3}, boff[3] = {s->off_b1, s->off_b2, s->off_b3};
     bf16 *wb[3] = {s->W1b, s->W2b, s->W3b};
     long long weights = 0;
-    int warps = 1;  // the loss
+    f.bias_blocks = 1;  // the loss
     for (int k = 0; k < 3; ++k) {
         f.wpart[k] = parts[k];
         f.wstride[k] = (long long)jobs[k]->zrows * jobs[k]->N;
@@ -629,13 +672,12 @@ tt_fsi_status step(tt_fsi_student_s *s, const float *x, const float *labels, con
         f.bn[k] = k == 2 ? s->n_out : s->H;
         f.boff[k] = boff[k];
         weights += f.wn[k];
-        warps += (f.bn[k] + 31) / 32;
+        f.bias_blocks += (f.bn[k] + 31) / 32;
     }
     f.loss_part = s->loss_part;
     f.loss_parts = pblocks;
     f.loss_scale = 1.0f / ((float)B * s->n_out);
     f.loss = loss_dev;
-    f.bias_blocks = (warps + 7) / 8;
     f.update = update;
     if (update) {
         s->step += 1;
@@ -705,7 +747,7 @@ tt_fsi_status tt_fsi_student_create(int d, int hidden, int n_out, int max_batch,
     A(&s->dYb, Bm * s->n_pad);
     A(&s->dH2, Bm * H);
     A(&s->dH1, Bm * H);
-    const size_t mtiles = (Bm + ttfsi_gemm::BM - 1) / ttfsi_gemm::BM, pblocks = (Bm + 8 * kTrainRows - 1) / (8 * kTrainRows);
+    const size_t mtiles = (Bm + ttfsi_gemm::BM - 1) / ttfsi_gemm::BM, pblocks = (Bm + kProjectRows - 1) / kProjectRows;
     A(&s->col1, mtiles * H);
     A(&s->col2, mtiles * H);
     A(&s->col3, pblocks * n_out);
@@ -739,7 +781,7 @@ tt_fsi_status tt_fsi_student_create(int d, int hidden, int n_out, int max_batch,
     tt_fsi_status r = st_status(e);
     if (r == TT_FSI_OK)
         r = st_status(cudaFuncSetAttribute(ttfsi_sgemm::student_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           ttfsi_sgemm::SG_SMEM));
+                                           ttfsi_sgemm::sg_smem(ttfsi_sgemm::SG_MAX_STAGES)));
     if (r == TT_FSI_OK) r = refresh_bf16(s, nullptr);
     if (r == TT_FSI_OK) r = st_status(cudaDeviceSynchronize());
     if (r != TT_FSI_OK) {
@@ -794,7 +836,7 @@ tt_fsi_status tt_fsi_student_predict(tt_fsi_student s, const float *x_dev, const
     if (r != TT_FSI_OK) return r;
     ttfsi_student::ProjectArgs p = project_args(s, target_dev, v_empty, B);
     p.phi = phi_dev;
-    return chain(ttfsi_student::project_kernel<1>, (unsigned)((B + 7) / 8), 256, 0, st, p);
+    return chain(ttfsi_student::project_kernel, (unsigned)((B + kProjectRows - 1) / kProjectRows), 256, 0, st, p);
 }
 
 tt_fsi_status tt_fsi_student_get_state(tt_fsi_student s, float *params_host, float *adam_m_host, float *adam_v_host,

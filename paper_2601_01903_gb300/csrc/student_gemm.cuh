@@ -11,9 +11,10 @@
 // written and read back per step at 4096 x 1024).
 //
 // One CTA of 8 warps computes a 128 x 128 tile of one K slice: one thread
-// issues TMA loads into two 32 KB stages, one issues the MMAs, all warps run
-// the epilogue, each on 32 rows x 64 columns.  66 KB of shared memory and 85
-// registers keep three CTAs on an SM, whose epilogues and main loops overlap.
+// issues TMA loads into 32 KB stages, one issues the MMAs, all warps run
+// the epilogue, each on 32 rows x 64 columns.  Two stages and 85 registers
+// keep three CTAs on an SM, whose epilogues and main loops overlap; a launch
+// with fewer CTAs takes more stages.
 // The epilogue bounds these kernels (a tile of layer 2 is 64 k clocks of
 // tensor work for 96 KB of output): results go from registers through the
 // idle stages, in the swizzled order of a TMA store, and leave as whole lines;
@@ -32,9 +33,14 @@ namespace ttfsi_sgemm {
 
 using namespace ttfsi_gemm;
 
-constexpr int SG_STAGES = 2;
+constexpr int SG_MAX_STAGES = 6;  // of 32 KB
 constexpr int SG_THREADS = 256;
-constexpr int SG_SMEM = SG_STAGES * 2 * TILE_BYTES + 1024;
+constexpr int SG_SMS = 152;
+__host__ __device__ constexpr int sg_smem(int stages) { return stages * 2 * TILE_BYTES + 1024; }
+// A CTA's loads are bound by their latency (two stages in flight: a tile of 16
+// K blocks takes 14 us alone on its SM), so a launch takes as many stages as
+// fit with the CTAs per SM that it has.
+inline int sg_stages(int blocks) { return blocks <= SG_SMS ? 6 : blocks <= 2 * SG_SMS ? 3 : 2; }
 
 enum : int { kPartial = 0, kAct = 1, kDgelu = 2 };
 
@@ -60,6 +66,7 @@ struct Job {
 struct Jobs {
     Job j[2];
     int *err;
+    int stages;  // sg_stages
 };
 
 __device__ __forceinline__ void tma_store_2d(const void *tmap, uint32_t src, int x, int y) {
@@ -85,6 +92,73 @@ __device__ __forceinline__ float4 ld_shared4(uint32_t a) {
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<const uint32_t *>(&p);
+}
+
+// ---- GELU and its derivative of packed FP32 pairs: the formula of
+// normal_cdf_pdf, half its instructions ----
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pack2(float a, float b) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f2 v, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 both(float c) { return pack2(c, c); }
+
+// q = erfc(|z| / sqrt 2) / 2 and e = exp(-z^2 / 2)
+__device__ __forceinline__ void normal_tail2(f2 z, f2 &q, f2 &e) {
+    const f2 x = mul2(z & 0x7fffffff7fffffffull, both(0.70710678118654752f));
+    float a, b;
+    unpack2(fma2(both(0.3275911f), x, both(1.0f)), a, b);
+    asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(a));
+    asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(b));
+    const f2 t = pack2(a, b);
+    f2 p = fma2(both(0.5f * 1.061405429f), t, both(0.5f * -1.453152027f));
+    p = fma2(p, t, both(0.5f * 1.421413741f));
+    p = fma2(p, t, both(0.5f * -0.284496736f));
+    p = fma2(p, t, both(0.5f * 0.254829592f));
+    unpack2(mul2(mul2(x, x), both(-1.4426950408889634f)), a, b);
+    asm("ex2.approx.ftz.f32 %0, %0;" : "+f"(a));
+    asm("ex2.approx.ftz.f32 %0, %0;" : "+f"(b));
+    e = pack2(a, b);
+    q = mul2(mul2(p, t), e);
+}
+
+__device__ __forceinline__ f2 normal_cdf2(float z0, float z1, f2 q) {
+    float q0, q1;
+    unpack2(q, q0, q1);
+    return pack2(z0 >= 0.f ? 1.0f - q0 : q0, z1 >= 0.f ? 1.0f - q1 : q1);
+}
+
+// z Phi(z), rounded to BF16
+__device__ __forceinline__ uint32_t gelu_pair(float z0, float z1) {
+    const f2 z = pack2(z0, z1);
+    f2 q, e;
+    normal_tail2(z, q, e);
+    float y0, y1;
+    unpack2(mul2(z, normal_cdf2(z0, z1, q)), y0, y1);
+    return pack_bf16(y0, y1);
+}
+
+// v0, v1 times d/dz [z Phi(z)] = Phi(z) + z phi(z)
+__device__ __forceinline__ void scale_gelu_grad(float &v0, float &v1, float z0, float z1) {
+    const f2 z = pack2(z0, z1);
+    f2 q, e;
+    normal_tail2(z, q, e);
+    const f2 pdf = mul2(both(0.39894228040143268f), e);
+    unpack2(mul2(pack2(v0, v1), fma2(z, pdf, normal_cdf2(z0, z1, q))), v0, v1);
 }
 
 // 32 accumulator columns of the lane's row.
@@ -123,7 +197,7 @@ __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.laun
 __global__ void __launch_bounds__(SG_THREADS, 3) student_gemm_kernel(const __grid_constant__ Jobs jobs) {
     extern __shared__ __align__(1024) unsigned char sg_raw[];
     const uint32_t base = (smem_u32(sg_raw) + 1023) & ~1023u;
-    __shared__ __align__(8) uint64_t full[SG_STAGES], empty[SG_STAGES], done, zbar[8];
+    __shared__ __align__(8) uint64_t full[SG_MAX_STAGES], empty[SG_MAX_STAGES], done, zbar[8];
     __shared__ uint32_t tmem_base_sh;
     __shared__ int s_fail;
     __shared__ float red[4][BN];
@@ -141,7 +215,7 @@ __global__ void __launch_bounds__(SG_THREADS, 3) student_gemm_kernel(const __gri
     const int n_cols = min(BN, a.N - n0);
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < SG_STAGES; ++s) {
+        for (int s = 0; s < jobs.stages; ++s) {
             mbar_init(smem_u32(&full[s]), 1);
             mbar_init(smem_u32(&empty[s]), 1);
         }
@@ -170,10 +244,9 @@ __global__ void __launch_bounds__(SG_THREADS, 3) student_gemm_kernel(const __gri
             // producer; the second half of an MN-major B tile is loaded only where columns use it
             const bool b_one = a.b_mn && n_cols <= 64;
             const uint32_t bytes = (b_one ? TILE_BYTES / 2 : TILE_BYTES) + TILE_BYTES;
-            int kb = 0;
-            for (; kb < nk; ++kb) {
-                const int s = kb % SG_STAGES;
-                const uint32_t use = (uint32_t)(kb / SG_STAGES);
+            int kb = 0, s = 0;
+            uint32_t use = 0;
+            for (; kb < nk; ++kb, use += ++s == jobs.stages, s = s == jobs.stages ? 0 : s) {
                 if (use > 0 && !mbar_wait(smem_u32(&empty[s]), (use - 1) & 1u)) {
                     atomicOr(&s_fail, 1);
                     break;
@@ -196,8 +269,8 @@ __global__ void __launch_bounds__(SG_THREADS, 3) student_gemm_kernel(const __gri
                 }
             }
             if (kb < nk)  // gave up: let the loads in flight land before the CTA ends
-                for (int i = max(0, kb - SG_STAGES); i < kb; ++i)
-                    mbar_wait(smem_u32(&full[i % SG_STAGES]), (uint32_t)(i / SG_STAGES) & 1u);
+                for (int i = max(0, kb - jobs.stages); i < kb; ++i)
+                    mbar_wait(smem_u32(&full[i % jobs.stages]), (uint32_t)(i / jobs.stages) & 1u);
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -207,9 +280,10 @@ __global__ void __launch_bounds__(SG_THREADS, 3) student_gemm_kernel(const __gri
                                    ((uint32_t)a.b_mn << 16);
             const uint32_t stepA = a.a_mn ? 2048u : 32u, stepB = a.b_mn ? 2048u : 32u;
             bool ok = true;
-            for (int kb = 0; kb < nk; ++kb) {
-                const int s = kb % SG_STAGES;
-                if (!mbar_wait(smem_u32(&full[s]), (uint32_t)(kb / SG_STAGES) & 1u)) {
+            int s = 0;
+            uint32_t use = 0;
+            for (int kb = 0; kb < nk; ++kb, use += ++s == jobs.stages, s = s == jobs.stages ? 0 : s) {
+                if (!mbar_wait(smem_u32(&full[s]), use & 1u)) {
                     ok = false;
                     break;
                 }
@@ -285,7 +359,7 @@ __global__ void __launch_bounds__(SG_THREADS, 3) student_gemm_kernel(const __gri
                         if (lane == 0) tma_store_2d(&a.F, buf + j * 4096, col0 + 32 * j, row0);
                     }
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) y[16 * j + i] = pack_bf16(gelu_f(v[2 * i]), gelu_f(v[2 * i + 1]));
+                    for (int i = 0; i < 16; ++i) y[16 * j + i] = gelu_pair(v[2 * i], v[2 * i + 1]);
                 } else {
 #pragma unroll
                     for (int i = 0; i < 16; ++i) y[16 * j + i] = 0u;
@@ -322,10 +396,8 @@ __global__ void __launch_bounds__(SG_THREADS, 3) student_gemm_kernel(const __gri
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
                     const float4 z = ld_shared4(line + j * 4096 + ((c ^ sw) << 4));
-                    v[4 * c] *= gelu_grad_f(z.x);
-                    v[4 * c + 1] *= gelu_grad_f(z.y);
-                    v[4 * c + 2] *= gelu_grad_f(z.z);
-                    v[4 * c + 3] *= gelu_grad_f(z.w);
+                    scale_gelu_grad(v[4 * c], v[4 * c + 1], z.x, z.y);
+                    scale_gelu_grad(v[4 * c + 2], v[4 * c + 3], z.z, z.w);
                 }
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
