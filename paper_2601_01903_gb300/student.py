@@ -230,6 +230,9 @@ class Explainer:
     def _values_listed(self, x64, c, out, tc):
         if tc:
             return masked_game_tc(self.mlp, x64, self.baseline, coalitions=c, out=out)
+        return self._values_listed_f32(x64, c, out)
+
+    def _values_listed_f32(self, x64, c, out):
         _check(_declare().tt_fsi_masked_game_sampled(ctypes.byref(self.mlp.struct), _p(x64), _p(self.baseline),
                                                       x64.shape[0], _p(c), c.shape[1], _p(out), _stream_ptr()),
                "tt_fsi_masked_game_sampled")
@@ -309,14 +312,28 @@ class Explainer:
         lib = _declare()
         n = x32.shape[0]
         r = torch.empty(n, dtype=torch.float32, device="cuda")
-        x64 = x32.double()
+        x64 = x32.to(device="cuda", dtype=torch.float64).contiguous()
+        # The chunks are queued without a look at the kernels' error flag in
+        # between (which idled the GPU for as long as a chunk of 2000 takes);
+        # they share one flag, read once before the residuals are returned.
+        err = torch.zeros(1, dtype=torch.int32, device="cuda")
+        vcoal = torch.empty((min(n, self.batch), self.K), dtype=torch.float32, device="cuda")
+        base = self.baseline.contiguous()
+        n_bg = 1 if base.dim() == 1 else base.shape[0]
+        stream = _stream_ptr()
         for s in range(0, n, self.batch):
             e = min(n, s + self.batch)
             c = self.coal_pool_dev[:e - s]
-            vcoal = torch.empty(c.shape, dtype=torch.float32, device="cuda")
-            self._values_listed(x64[s:e], c, vcoal, self.tc)
+            if self.tc:
+                _check(lib.tt_fsi_masked_game_tc_interventional(
+                    ctypes.byref(self.mlp.struct), _p(x64[s:e]), _p(base), n_bg, e - s, _p(c), self.K, _p(vcoal),
+                    _p(err), stream), "tt_fsi_masked_game_tc_interventional")
+            else:
+                self._values_listed_f32(x64[s:e], c, vcoal[:e - s])
             _check(lib.tt_fsi_surrogate_residual(_p(phi[s:e]), e - s, self.n_out, _p(self.masks), _p(c), _p(vcoal),
-                                                  self.K, _p(r[s:e]), _stream_ptr()), "tt_fsi_surrogate_residual")
+                                                  self.K, _p(r[s:e]), stream), "tt_fsi_surrogate_residual")
+        if self.tc and int(err.item()) != 0:
+            raise FsiError(5, "tt_fsi_masked_game_tc")
         return r
 
     def calibrate(self, data: Dataset, quantile: float = 0.99):
