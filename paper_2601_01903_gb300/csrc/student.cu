@@ -535,7 +535,19 @@ bool out_dgelu(ttfsi_sgemm::Job &j, const float *Z, bf16 *Hb, float *colpart) {
     j.kind = ttfsi_sgemm::kDgelu;
     j.colpart = colpart;
     return encode_map(&j.Z, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, Z, j.M, j.N, j.N, 32, 32) &&
-           encode_map(&j.Hb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Hb, j.M, j.N, j.N, 64, 32);
+           (!Hb || encode_map(&j.Hb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Hb, j.M, j.N, j.N, 64, 32));
+}
+
+// dH1's product also forms its tile's part of dW1 = dH1^T X where a row of X
+// fits one box (otherwise dH1 is written out and dW1 has a launch of its own;
+// 4096 x 1024, d = 16: 92.6 us a step with it, 97.2 us without).
+bool dw1_fused(const tt_fsi_student_s *s) { return s->d <= 64; }
+
+bool out_dw(ttfsi_sgemm::Job &j, const bf16 *X, int d, float *dwpart) {
+    j.dwx = 1;
+    j.xd = d;
+    j.dwpart = dwpart;
+    return encode_map(&j.X, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, X, j.M, d, d, 64, ttfsi_gemm::BM);
 }
 
 // The products for batches of B instances; made again when B changes.
@@ -568,7 +580,10 @@ tt_fsi_status plan_batch(tt_fsi_student_s *s, int B) {
          make_job(s->b2.j[1], s->dH2, H, 0, s->W2b, H, 1, B, H, H, false) &&
          out_dgelu(s->b2.j[1], s->Z1, s->dH1, s->col1);
     // dW1 = dH1^T X
-    ok = ok && make_job(s->b1.j[0], s->dH1, H, 1, s->Xb, d, 1, H, d, B, true) && out_partial(s->b1.j[0], s->part1, d);
+    if (dw1_fused(s))
+        ok = ok && out_dw(s->b2.j[1], s->Xb, d, s->part1);
+    else
+        ok = ok && make_job(s->b1.j[0], s->dH1, H, 1, s->Xb, d, 1, H, d, B, true) && out_partial(s->b1.j[0], s->part1, d);
     if (!ok) return TT_FSI_ERR_CUDA;
     for (auto *j : {&s->f1_train, &s->f1, &s->f2_train, &s->f2, &s->f3, &s->b3, &s->b2, &s->b1})
         j->stages = ttfsi_sgemm::sg_stages(j->j[0].blocks + j->j[1].blocks);
@@ -646,7 +661,7 @@ tt_fsi_status step(tt_fsi_student_s *s, const float *x, const float *labels, con
     r = chain(ttfsi_student::project_kernel, (unsigned)pblocks, 256, 0, st, p);
     if (r == TT_FSI_OK) r = run_jobs(s->b3, st);
     if (r == TT_FSI_OK) r = run_jobs(s->b2, st);
-    if (r == TT_FSI_OK) r = run_jobs(s->b1, st);
+    if (r == TT_FSI_OK && !dw1_fused(s)) r = run_jobs(s->b1, st);
     if (r != TT_FSI_OK) return r;
 
     ttfsi_student::FinishArgs f{};
@@ -662,10 +677,15 @@ tt_fsi_status step(tt_fsi_student_s *s, const float *x, const float *labels, con
     f.bias_blocks = 1;  // the loss
     for (int k = 0; k < 3; ++k) {
         f.wpart[k] = parts[k];
-        f.wstride[k] = (long long)jobs[k]->zrows * jobs[k]->N;
-        f.wslices[k] = job_slices(*jobs[k]);
+        if (k == 0 && dw1_fused(s)) {
+            f.wslices[k] = mtiles;
+            f.wn[k] = f.wstride[k] = (long long)s->H * s->d;
+        } else {
+            f.wslices[k] = job_slices(*jobs[k]);
+            f.wn[k] = (long long)jobs[k]->M * jobs[k]->N;
+            f.wstride[k] = (long long)jobs[k]->zrows * jobs[k]->N;
+        }
         f.woff[k] = woff[k];
-        f.wn[k] = (long long)jobs[k]->M * jobs[k]->N;
         f.wb[k] = wb[k];
         f.bpart[k] = cols[k];
         f.bparts[k] = k == 2 ? pblocks : mtiles;
@@ -746,7 +766,7 @@ tt_fsi_status tt_fsi_student_create(int d, int hidden, int n_out, int max_batch,
     A(&s->Z2, Bm * H);
     A(&s->dYb, Bm * s->n_pad);
     A(&s->dH2, Bm * H);
-    A(&s->dH1, Bm * H);
+    if (!dw1_fused(s)) A(&s->dH1, Bm * H);
     const size_t mtiles = (Bm + ttfsi_gemm::BM - 1) / ttfsi_gemm::BM, pblocks = (Bm + kProjectRows - 1) / kProjectRows;
     A(&s->col1, mtiles * H);
     A(&s->col2, mtiles * H);
@@ -772,7 +792,7 @@ tt_fsi_status tt_fsi_student_create(int d, int hidden, int n_out, int max_batch,
             for (int k = 0; k < 3; ++k) w[k] = std::max(w[k], rows(shape[k][0], shape[k][1], b));
         }
         A(&s->Y, y * s->ldy);
-        A(&s->part1, w[0] * d);
+        A(&s->part1, dw1_fused(s) ? mtiles * H * d : w[0] * d);
         A(&s->part2, w[1] * H);
         A(&s->part3, w[2] * H);
     }

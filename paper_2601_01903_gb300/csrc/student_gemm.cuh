@@ -47,17 +47,23 @@ enum : int { kPartial = 0, kAct = 1, kDgelu = 2 };
 // One product.  kPartial: the raw FP32 tile of K slice z goes to rows
 // z zrows .. of F.  kAct: z = acc + bias, F = z (when has_f), Hb = BF16
 // GELU(z).  kDgelu: g = acc gelu'(Z), Hb = BF16 g, and the column sums of g
-// over the tile's rows go to colpart[m tile][N].
+// over the tile's rows go to colpart[m tile][N].  With dwx, kDgelu multiplies
+// the tile, as it lies in shared memory, by its rows of X (a second product on
+// the tensor cores) and writes dwpart[m tile][N][xd], the tile's part of the
+// weight gradient below; g itself then stays on the chip.
 struct Job {
     CUtensorMap A, B;  // boxes of 64 x 128 (K-major) or 64 x 64 (MN-major) elements
     CUtensorMap F;     // FP32 output, boxes of 32 x 32
     CUtensorMap Hb;    // BF16 output, boxes of 64 x 32
     CUtensorMap Z;     // FP32 pre-activations, boxes of 32 x 32
+    CUtensorMap X;     // BF16 instances [M, xd], boxes of 64 x 128
     const float *bias;
     float *colpart;
     int M, N, K;
     int a_mn, b_mn;
     int kind, has_f;
+    int dwx, xd;  // xd: a multiple of 8, at most 64
+    float *dwpart;
     int kbc;     // K blocks of 64 per slice
     int zrows;   // rows between slices of F, a multiple of 32 no less than M rounded up to 32
     int tiles_n, tiles_m;
@@ -74,6 +80,10 @@ __device__ __forceinline__ void tma_store_2d(const void *tmap, uint32_t src, int
                  "r"(y), "r"(src)
                  : "memory");
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+
+__device__ __forceinline__ void prefetch_map(const CUtensorMap *m) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
 }
 
 __device__ __forceinline__ void st_shared4(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
@@ -179,12 +189,12 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
 
 // Shared-memory descriptor of an MN-major operand, 128-byte swizzle: 64
 // elements of M or N by 8 of K per 1024-byte group; the next 8 of K follow
-// (stride byte offset), the next 64 of M or N start 8192 bytes on (leading
+// (stride byte offset), the next 64 of M or N start `next` bytes on (leading
 // byte offset; one 64 x 64 box each).
-__device__ __forceinline__ uint64_t smem_desc_mn(uint32_t addr) {
+__device__ __forceinline__ uint64_t smem_desc_mn(uint32_t addr, uint32_t next = 8192) {
     uint64_t d = 0;
     d |= (uint64_t)((addr & 0x3FFFF) >> 4);
-    d |= (uint64_t)(8192 >> 4) << 16;
+    d |= (uint64_t)(next >> 4) << 16;
     d |= (uint64_t)(1024 >> 4) << 32;
     d |= (uint64_t)1 << 46;
     d |= (uint64_t)2 << 61;
@@ -197,7 +207,7 @@ __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.laun
 __global__ void __launch_bounds__(SG_THREADS, 3) student_gemm_kernel(const __grid_constant__ Jobs jobs) {
     extern __shared__ __align__(1024) unsigned char sg_raw[];
     const uint32_t base = (smem_u32(sg_raw) + 1023) & ~1023u;
-    __shared__ __align__(8) uint64_t full[SG_MAX_STAGES], empty[SG_MAX_STAGES], done, zbar[8];
+    __shared__ __align__(8) uint64_t full[SG_MAX_STAGES], empty[SG_MAX_STAGES], done, zbar[8], xbar, xdone;
     __shared__ uint32_t tmem_base_sh;
     __shared__ int s_fail;
     __shared__ float red[4][BN];
@@ -221,8 +231,16 @@ __global__ void __launch_bounds__(SG_THREADS, 3) student_gemm_kernel(const __gri
         }
         mbar_init(smem_u32(&done), 1);
         for (int w = 0; w < 8; ++w) mbar_init(smem_u32(&zbar[w]), 1);
+        mbar_init(smem_u32(&xbar), 1);
+        mbar_init(smem_u32(&xdone), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         s_fail = 0;
+    }
+    if (threadIdx.x == 64) {  // the descriptors, ahead of their first use
+        prefetch_map(&a.A);
+        prefetch_map(&a.B);
+        if (a.kind == kDgelu) prefetch_map(&a.Z);
+        prefetch_map(a.kind == kPartial ? &a.F : a.dwx ? &a.X : &a.Hb);
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_sh)),
@@ -306,11 +324,12 @@ __global__ void __launch_bounds__(SG_THREADS, 3) student_gemm_kernel(const __gri
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
     // Epilogue.  Warp w: rows 32 (w & 3) .., columns 64 (w >> 2) .., through
-    // its own 8 KB of the idle stages (two 32 x 128-byte blocks; row r's
-    // 16-byte chunk c at chunk c ^ (r & 7), the order of a 128-byte-swizzled
+    // its own 8 KB of the idle stages (two 32 x 128-byte blocks, 32 KB apart; row
+    // r's 16-byte chunk c at chunk c ^ (r & 7), the order of a 128-byte-swizzled
     // TMA copy).  A lane touches its own row only, so no lane waits for another.
+    constexpr uint32_t kNext = 32768;
     const int q = warp & 3, row0 = m0 + 32 * q, colw = 64 * (warp >> 2);
-    const uint32_t buf = base + (uint32_t)warp * 8192;
+    const uint32_t buf = base + (uint32_t)warp * 4096;
     const uint32_t line = buf + (uint32_t)lane * 128;
     const uint32_t sw = (uint32_t)(lane & 7);
     const bool fail = s_fail != 0;
@@ -325,11 +344,11 @@ __global__ void __launch_bounds__(SG_THREADS, 3) student_gemm_kernel(const __gri
                 tmem_ld32(trow + 32 * j, v);
 #pragma unroll
                 for (int c = 0; c < 8; ++c)
-                    st_shared4(line + j * 4096 + ((c ^ sw) << 4), __float_as_uint(v[4 * c]), __float_as_uint(v[4 * c + 1]),
+                    st_shared4(line + j * kNext + ((c ^ sw) << 4), __float_as_uint(v[4 * c]), __float_as_uint(v[4 * c + 1]),
                                __float_as_uint(v[4 * c + 2]), __float_as_uint(v[4 * c + 3]));
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
-                if (lane == 0) tma_store_2d(&a.F, buf + j * 4096, col0 + 32 * j, slice * a.zrows + row0);
+                if (lane == 0) tma_store_2d(&a.F, buf + j * kNext, col0 + 32 * j, slice * a.zrows + row0);
             }
         } else if (kind == kAct) {
             uint32_t y[32];
@@ -351,12 +370,12 @@ __global__ void __launch_bounds__(SG_THREADS, 3) student_gemm_kernel(const __gri
                     if (a.has_f) {
 #pragma unroll
                         for (int c = 0; c < 8; ++c)
-                            st_shared4(line + j * 4096 + ((c ^ sw) << 4), __float_as_uint(v[4 * c]),
+                            st_shared4(line + j * kNext + ((c ^ sw) << 4), __float_as_uint(v[4 * c]),
                                        __float_as_uint(v[4 * c + 1]), __float_as_uint(v[4 * c + 2]),
                                        __float_as_uint(v[4 * c + 3]));
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         __syncwarp();
-                        if (lane == 0) tma_store_2d(&a.F, buf + j * 4096, col0 + 32 * j, row0);
+                        if (lane == 0) tma_store_2d(&a.F, buf + j * kNext, col0 + 32 * j, row0);
                     }
 #pragma unroll
                     for (int i = 0; i < 16; ++i) y[16 * j + i] = gelu_pair(v[2 * i], v[2 * i + 1]);
@@ -383,7 +402,7 @@ __global__ void __launch_bounds__(SG_THREADS, 3) student_gemm_kernel(const __gri
             const uint32_t bar = smem_u32(&zbar[warp]);
             if (lane == 0) {
                 mbar_expect_tx(bar, 4096u * (uint32_t)nj);
-                for (int j = 0; j < nj; ++j) tma_load_2d(buf + j * 4096, &a.Z, col0 + 32 * j, row0, bar);
+                for (int j = 0; j < nj; ++j) tma_load_2d(buf + j * kNext, &a.Z, col0 + 32 * j, row0, bar);
             }
             __syncwarp();
             const bool ok = mbar_wait(bar, 0);
@@ -395,7 +414,7 @@ __global__ void __launch_bounds__(SG_THREADS, 3) student_gemm_kernel(const __gri
                 // replace chunks 4 j .. of the first block, which half 0 has read
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
-                    const float4 z = ld_shared4(line + j * 4096 + ((c ^ sw) << 4));
+                    const float4 z = ld_shared4(line + j * kNext + ((c ^ sw) << 4));
                     scale_gelu_grad(v[4 * c], v[4 * c + 1], z.x, z.y);
                     scale_gelu_grad(v[4 * c + 2], v[4 * c + 3], z.z, z.w);
                 }
@@ -418,18 +437,58 @@ __global__ void __launch_bounds__(SG_THREADS, 3) student_gemm_kernel(const __gri
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
-            if (lane == 0 && ok) tma_store_2d(&a.Hb, buf, col0, row0);
+            if (lane == 0 && ok && !a.dwx) tma_store_2d(&a.Hb, buf, col0, row0);
         }
     }
     if (!fail && kind == kDgelu) {
         if (row0 >= a.M) {
             red[q][colw + lane] = 0.0f;
             red[q][colw + 32 + lane] = 0.0f;
+            if (a.dwx) {
+#pragma unroll
+                for (int c = 0; c < 8; ++c) st_shared4(line + (c << 4), 0u, 0u, 0u, 0u);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            }
         }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
+        if (a.dwx && threadIdx.x == 0) {
+            // g^T X: the first blocks are the tile [128 rows][2 x 64 columns],
+            // MN-major; X replaces the second ones, all read by now
+            const uint32_t xs = base + kNext;
+            mbar_expect_tx(smem_u32(&xbar), TILE_BYTES);
+            tma_load_2d(xs, &a.X, 0, m0, smem_u32(&xbar));
+            const bool ok = mbar_wait(smem_u32(&xbar), 0);
+            if (!ok) atomicOr(jobs.err, kErrGemmTimeout);
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t idesc = instr_desc_bf16(BM, (a.xd + 15) & ~15) | (1u << 15) | (1u << 16);
+            if (ok)
+                for (int k16 = 0; k16 < BM / 16; ++k16)
+                    mma_bf16(tmem, smem_desc_mn(base + k16 * 2048, 16384), smem_desc_mn(xs + k16 * 2048), idesc,
+                             k16 > 0 ? 1u : 0u);
+            mma_commit(smem_u32(&xdone));
+        }
         if ((int)threadIdx.x < n_cols)
             a.colpart[(long long)(m0 / BM) * a.N + n0 + threadIdx.x] =
                 (red[0][threadIdx.x] + red[1][threadIdx.x]) + (red[2][threadIdx.x] + red[3][threadIdx.x]);
+        __syncwarp();
+        if (a.dwx && warp < 4) {
+            if (!mbar_wait(smem_u32(&xdone), 0) && lane == 0) atomicOr(jobs.err, kErrGemmTimeout);
+            __syncwarp();
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const int h = n0 + 32 * warp + lane;
+            float *out = a.dwpart + ((long long)(m0 / BM) * a.N + h) * a.xd;
+            for (int c0 = 0; c0 < a.xd; c0 += 32) {
+                float v[32];
+                tmem_ld32(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0, v);
+                if (h < a.N)
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        if (c0 + 4 * c < a.xd)
+                            *reinterpret_cast<float4 *>(out + c0 + 4 * c) =
+                                make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+            }
+        }
     }
     if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
