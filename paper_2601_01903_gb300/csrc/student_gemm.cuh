@@ -82,6 +82,13 @@ __device__ __forceinline__ void tma_store_2d(const void *tmap, uint32_t src, int
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
+// One lane of a converged warp, the same at every call.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ void prefetch_map(const CUtensorMap *m) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
 }
@@ -257,63 +264,86 @@ __global__ void __launch_bounds__(SG_THREADS, 3) student_gemm_kernel(const __gri
     auto tileA = [&](int s) { return base + (uint32_t)(s * 2) * TILE_BYTES; };
     auto tileB = [&](int s) { return base + (uint32_t)(s * 2 + 1) * TILE_BYTES; };
 
+    // Warps 0 and 1 go through their loops whole and elect one lane for each
+    // copy or MMA: the operands stay in uniform registers, where a branch on
+    // the lane makes the compiler move them there under divergence (a K block
+    // took 900 clocks of issue, 256 of tensor work).
     if (warp == 0) {
-        if (lane == 0) {
-            // producer; the second half of an MN-major B tile is loaded only where columns use it
-            const bool b_one = a.b_mn && n_cols <= 64;
-            const uint32_t bytes = (b_one ? TILE_BYTES / 2 : TILE_BYTES) + TILE_BYTES;
-            int kb = 0, s = 0;
-            uint32_t use = 0;
-            for (; kb < nk; ++kb, use += ++s == jobs.stages, s = s == jobs.stages ? 0 : s) {
-                if (use > 0 && !mbar_wait(smem_u32(&empty[s]), (use - 1) & 1u)) {
-                    atomicOr(&s_fail, 1);
-                    break;
-                }
-                if (*(volatile int *)&s_fail) break;
+        // producer; an operand tile is two halves of 64 rows (or columns), 8 KB each,
+        // the second half of B only where columns use it
+        const bool b_one = a.b_mn && n_cols <= 64;
+        const uint32_t bytes = (b_one ? TILE_BYTES / 2 : TILE_BYTES) + TILE_BYTES;
+        const bool leader = elect_one();
+        const int a_mn = a.a_mn, b_mn = a.b_mn, stages = jobs.stages;
+        int kb = 0, s = 0;
+        uint32_t use = 0;
+        for (; kb < nk; ++kb) {
+            if (use > 0 && !mbar_wait(smem_u32(&empty[s]), (use - 1) & 1u)) {
+                if (leader) atomicOr(&s_fail, 1);
+                break;
+            }
+            if (leader) {
                 const uint32_t bar = smem_u32(&full[s]);
                 mbar_expect_tx(bar, bytes);
                 const int k0 = (kb0 + kb) * BK;
-                if (a.a_mn) {
-                    tma_load_2d(tileA(s), &a.A, m0, k0, bar);
-                    tma_load_2d(tileA(s) + TILE_BYTES / 2, &a.A, m0 + 64, k0, bar);
+                const uint32_t ta = tileA(s), tb = tileB(s);
+                if (a_mn) {
+                    tma_load_2d(ta, &a.A, m0, k0, bar);
+                    tma_load_2d(ta + TILE_BYTES / 2, &a.A, m0 + 64, k0, bar);
                 } else {
-                    tma_load_2d(tileA(s), &a.A, k0, m0, bar);
+                    tma_load_2d(ta, &a.A, k0, m0, bar);
                 }
-                if (a.b_mn) {
-                    tma_load_2d(tileB(s), &a.B, n0, k0, bar);
-                    if (!b_one) tma_load_2d(tileB(s) + TILE_BYTES / 2, &a.B, n0 + 64, k0, bar);
+                if (b_mn) {
+                    tma_load_2d(tb, &a.B, n0, k0, bar);
+                    if (!b_one) tma_load_2d(tb + TILE_BYTES / 2, &a.B, n0 + 64, k0, bar);
                 } else {
-                    tma_load_2d(tileB(s), &a.B, k0, n0, bar);
+                    tma_load_2d(tb, &a.B, k0, n0, bar);
                 }
             }
-            if (kb < nk)  // gave up: let the loads in flight land before the CTA ends
-                for (int i = max(0, kb - jobs.stages); i < kb; ++i)
-                    mbar_wait(smem_u32(&full[i % jobs.stages]), (uint32_t)(i / jobs.stages) & 1u);
+            __syncwarp();
+            if (++s == stages) {
+                s = 0;
+                ++use;
+            }
         }
+        if (kb < nk)  // gave up: let the loads in flight land before the CTA ends
+            for (int i = max(0, kb - stages); i < kb; ++i)
+                mbar_wait(smem_u32(&full[i % stages]), (uint32_t)(i / stages) & 1u);
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            // MMA issuer: as many columns as the tile has, in sixteens
-            const uint32_t idesc = instr_desc_bf16(BM, (n_cols + 15) & ~15) | ((uint32_t)a.a_mn << 15) |
-                                   ((uint32_t)a.b_mn << 16);
-            const uint32_t stepA = a.a_mn ? 2048u : 32u, stepB = a.b_mn ? 2048u : 32u;
-            bool ok = true;
-            int s = 0;
-            uint32_t use = 0;
-            for (int kb = 0; kb < nk; ++kb, use += ++s == jobs.stages, s = s == jobs.stages ? 0 : s) {
-                if (!mbar_wait(smem_u32(&full[s]), use & 1u)) {
-                    ok = false;
-                    break;
-                }
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const int steps = min(BK / 16, (a.K - (kb0 + kb) * BK + 15) / 16);
-                for (int k16 = 0; k16 < steps; ++k16) {
-                    const uint32_t pa = tileA(s) + k16 * stepA, pb = tileB(s) + k16 * stepB;
-                    mma_bf16(tmem, a.a_mn ? smem_desc_mn(pa) : smem_desc(pa), a.b_mn ? smem_desc_mn(pb) : smem_desc(pb),
-                             idesc, (kb > 0 || k16 > 0) ? 1u : 0u);
-                }
+        // MMA issuer: as many columns as the tile has, in sixteens (K beyond the
+        // operands was filled with zeros)
+        const uint32_t idesc =
+            instr_desc_bf16(BM, (n_cols + 15) & ~15) | ((uint32_t)a.a_mn << 15) | ((uint32_t)a.b_mn << 16);
+        const uint32_t stepA = (a.a_mn ? 2048u : 32u) >> 4, stepB = (a.b_mn ? 2048u : 32u) >> 4;
+        const uint64_t da0 = a.a_mn ? smem_desc_mn(tileA(0)) : smem_desc(tileA(0));
+        const uint64_t db0 = a.b_mn ? smem_desc_mn(tileB(0)) : smem_desc(tileB(0));
+        const int stages = jobs.stages;
+        const bool leader = elect_one();
+        bool ok = true;
+        int s = 0;
+        uint32_t parity = 0;
+        for (int kb = 0; kb < nk; ++kb) {
+            if (!mbar_wait(smem_u32(&full[s]), parity)) {
+                ok = false;
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if (leader) {
+                const uint64_t da = da0 + (uint32_t)(s * (2 * TILE_BYTES >> 4));
+                const uint64_t db = db0 + (uint32_t)(s * (2 * TILE_BYTES >> 4));
+#pragma unroll
+                for (int k16 = 0; k16 < BK / 16; ++k16)
+                    mma_bf16(tmem, da + k16 * stepA, db + k16 * stepB, idesc, (kb > 0 || k16 > 0) ? 1u : 0u);
                 mma_commit(smem_u32(&empty[s]));
             }
+            __syncwarp();
+            if (++s == stages) {
+                s = 0;
+                parity ^= 1u;
+            }
+        }
+        if (leader) {
             if (!ok) atomicOr(&s_fail, 1);
             mma_commit(smem_u32(&done));  // arrives once every MMA issued above has completed
         }
