@@ -757,7 +757,7 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
             failed = true;
             break;
         }
-        if (tid == 0) {
+        if (warp == 0 && ttfsi_gemm::elect_one()) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int n_k16 = (min(KC, a.h1 - kc * KC) + 15) >> 4;
             const uint64_t da = smem_desc(a_base), dw = smem_desc(w_base + (F64 ? 0 : kc * (NS * NW * 128)));

@@ -82,13 +82,6 @@ __device__ __forceinline__ void tma_store_2d(const void *tmap, uint32_t src, int
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
-// One lane of a converged warp, the same at every call.
-__device__ __forceinline__ bool elect_one() {
-    uint32_t p;
-    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
-    return p != 0;
-}
-
 __device__ __forceinline__ void prefetch_map(const CUtensorMap *m) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
 }
@@ -219,7 +212,7 @@ __global__ void __launch_bounds__(SG_THREADS, 3) student_gemm_kernel(const __gri
     __shared__ int s_fail;
     __shared__ float red[4][BN];
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int which = (int)blockIdx.x >= jobs.j[0].blocks;
     const Job &a = jobs.j[which];
     int t = (int)blockIdx.x - (which ? jobs.j[0].blocks : 0);
