@@ -307,8 +307,8 @@ tt_fsi_status tt_fsi_batch_set_wait_limit(tt_fsi_batch batch, long long polls, i
 tt_fsi_status tt_fsi_batch_check(tt_fsi_batch batch, struct CUstream_st *stream);
 
 /*
- * BF16 GEMM on the tcgen05 tensor cores (the building block of the student
- * explainer; no counterpart in the paper's method, which has no learned part):
+ * BF16 GEMM on the tcgen05 tensor cores (no counterpart in the paper's method,
+ * which has no learned part):
  *   Z = A . B^T (+ bias) (* gelu'(dgelu_z) elementwise),  FP32 accumulation,
  *   A [M, K] and B [N, K] row-major BF16 device arrays (lda, ldb multiples of
  *   8 elements, >= K; 16-byte aligned), bias [N] FP32 or NULL,
@@ -326,9 +326,9 @@ tt_fsi_status tt_fsi_gemm_bf16(const void *A, int lda, const void *B, int ldb, i
 /*
  * Amortised explainer ("student").  No counterpart in the paper's method:
  * a GELU MLP x [d] -> H -> H -> n_out maps an instance straight to its FSI
- * scores, trained on (x, exact FSI of v_x) pairs.  Every GEMM of its forward
- * and backward passes runs on tt_fsi_gemm_bf16 (BF16 operands, FP32
- * accumulation); master weights and Adam state are FP32.  Its raw outputs
+ * scores, trained on (x, exact FSI of v_x) pairs.  Every matrix product of its
+ * forward and backward passes runs on the tcgen05 tensor cores (BF16 operands,
+ * FP32 accumulation); master weights and Adam state are FP32.  Its raw outputs
  * are projected onto the efficiency constraint: phi(empty) = v_empty and
  * the other n_out - 1 scores are shifted equally so that they sum to
  * target[b] = v_b(N) - v_empty.
