@@ -3,7 +3,7 @@
 // tensor cores (student_gemm.cuh).  A training step is eight launches: the
 // instances to BF16, three layers forward, the projection with loss and output
 // gradient, [dH2 | dW3], [dW2 | dH1 with dW1], and the sums of partial results
-// with Adam.  One GB300, 4096 instances, 1024 hidden units, 137 scores: 81.5 us
+// with Adam.  One GB300, 4096 instances, 1024 hidden units, 137 scores: 79 us
 // (0.236 ms with 20 launches, transposed copies and separate sums).  This file
 // also holds the launcher of the general BF16 GEMM (gemm_tcgen05.cuh) and its
 // C ABI entry point.
@@ -154,7 +154,10 @@ __global__ void to_bf16_kernel(CastJobs c) {
 // on the non-empty coordinates, 0 on the empty one, as BF16 (the operand of
 // the backward products), its FP32 column sums over the block's rows (the bias
 // gradient's partial sums) and the block's loss.  A warp takes a row, a block
-// 8; y is kept in the first slice's row, which only its own lanes read.
+// 8; the first 256 columns of y and the labels stay in registers over the three
+// passes, the rest of y in the first slice's row, which only its own lanes
+// read (a step of 4096 x 137 81.3 us with all of them re-read, 79.0 us so; bound by
+// the latency of its loads, 27 warps per SM in one wave).
 struct ProjectArgs {
     float *Y;  // [slices][zrows][ldy]
     int slices, ldy;
@@ -176,78 +179,118 @@ __device__ __forceinline__ float warp_sum(float s) {
 }
 
 __global__ void __launch_bounds__(256) project_kernel(const ProjectArgs a) {
-    constexpr int C = 4;  // columns per lane in flight
-    __shared__ float red[8][32 * C];
+    constexpr int C = 4, CW = 32 * C;  // columns per lane and per warp in flight
+    constexpr int KEEP = 2;            // chunks of CW columns held in registers
+    __shared__ float red[8][CW];
     __shared__ float lred[8];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row = blockIdx.x * 8 + warp, n_out = a.n_out;
     const bool in = row < a.B;
     ttfsi_sgemm::pdl_launch();
     ttfsi_sgemm::pdl_wait();
-    float *y = a.Y + (long long)(in ? row : 0) * a.ldy;
+    float *Y = a.Y + (long long)(in ? row : 0) * a.ldy;
     const long long at = (long long)(in ? row : 0) * n_out;
-    float sum = 0.f;
-    if (in)
-        for (int k0 = lane; k0 < n_out; k0 += 32 * C) {
-            float v[C] = {};
+    // columns k0 + 32 c of the row: raw outputs (the slices' sum plus the bias), labels
+    auto outputs = [&](int k0, float (&y)[C]) {
+#pragma unroll
+        for (int c = 0; c < C; ++c) y[c] = 0.f;
 #pragma unroll 4
-            for (int z = 0; z < a.slices; ++z)
+        for (int z = 0; z < a.slices; ++z)
 #pragma unroll
-                for (int c = 0; c < C; ++c) v[c] += y[z * a.zstride + min(k0 + 32 * c, n_out - 1)];
+            for (int c = 0; c < C; ++c) y[c] += Y[z * a.zstride + min(k0 + 32 * c, n_out - 1)];
 #pragma unroll
-            for (int c = 0; c < C; ++c) {
-                const int k = k0 + 32 * c;
-                if (k >= n_out) break;
-                v[c] += a.bias[k];
-                if (k > 0) sum += v[c];
-                y[k] = v[c];
+        for (int c = 0; c < C; ++c) y[c] += a.bias[min(k0 + 32 * c, n_out - 1)];
+    };
+    auto labels = [&](int k0, float (&l)[C]) {
+#pragma unroll
+        for (int c = 0; c < C; ++c) l[c] = a.labels ? a.labels[at + min(k0 + 32 * c, n_out - 1)] : 0.f;
+    };
+    auto kept_outputs = [&](int k0, float (&y)[C]) {
+#pragma unroll
+        for (int c = 0; c < C; ++c) y[c] = Y[min(k0 + 32 * c, n_out - 1)];
+    };
+
+    float yk[KEEP][C] = {}, lk[KEEP][C] = {};
+    float sum = 0.f;
+    auto add_outputs = [&](int k0, const float (&y)[C]) {
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+            if (k0 + 32 * c > 0 && k0 + 32 * c < n_out) sum += y[c];
+    };
+    if (in) {
+#pragma unroll
+        for (int h = 0; h < KEEP; ++h)
+            if (h * CW < n_out) {
+                outputs(h * CW + lane, yk[h]);
+                labels(h * CW + lane, lk[h]);
             }
+#pragma unroll
+        for (int h = 0; h < KEEP; ++h) add_outputs(h * CW + lane, yk[h]);
+        for (int k0 = KEEP * CW + lane; k0 < n_out; k0 += CW) {
+            float y[C];
+            outputs(k0, y);
+            add_outputs(k0, y);
+#pragma unroll
+            for (int c = 0; c < C; ++c)
+                if (k0 + 32 * c < n_out) Y[k0 + 32 * c] = y[c];
         }
+    }
     const float shift = in ? (a.target[row] - warp_sum(sum)) / (float)(n_out - 1) : 0.f;
     const float scale = 2.0f / ((float)a.B * (float)n_out);
     float loss = 0.f, gsum = 0.f;
-    if (in)
-        for (int k0 = lane; k0 < n_out; k0 += 32 * C) {
-            float p[C], l[C];
+    auto project = [&](int k0, const float (&y)[C], const float (&l)[C]) {
 #pragma unroll
-            for (int c = 0; c < C; ++c) {
-                const int k = min(k0 + 32 * c, n_out - 1);
-                p[c] = y[k];
-                l[c] = a.labels ? a.labels[at + k] : 0.f;
-            }
-#pragma unroll
-            for (int c = 0; c < C; ++c) {
-                const int k = k0 + 32 * c;
-                if (k >= n_out) break;
-                p[c] = (k == 0) ? a.v_empty : p[c] + shift;
-                if (a.phi) a.phi[at + k] = p[c];
-                const float e = p[c] - l[c];
-                loss += e * e;
-                if (k > 0) gsum += scale * e;
-            }
+        for (int c = 0; c < C; ++c) {
+            const int k = k0 + 32 * c;
+            if (k >= n_out) break;
+            const float p = (k == 0) ? a.v_empty : y[c] + shift;
+            if (a.phi) a.phi[at + k] = p;
+            const float e = p - l[c];
+            loss += e * e;
+            if (k > 0) gsum += scale * e;
         }
+    };
+    if (in) {
+#pragma unroll
+        for (int h = 0; h < KEEP; ++h) project(h * CW + lane, yk[h], lk[h]);
+        for (int k0 = KEEP * CW + lane; k0 < n_out; k0 += CW) {
+            float y[C], l[C];
+            kept_outputs(k0, y);
+            labels(k0, l);
+            project(k0, y, l);
+        }
+    }
     if (!a.labels) return;
     const float gmean = warp_sum(gsum) / (float)(n_out - 1);
     loss = warp_sum(loss);
     if (lane == 0) lred[warp] = loss;
-    for (int k1 = 0; k1 < a.ld_dyb; k1 += 32 * C) {
+    auto gradient = [&](int k1, const float (&y)[C], const float (&l)[C]) {
 #pragma unroll
         for (int c = 0; c < C; ++c) {
             const int k = k1 + 32 * c + lane;
             float g = 0.f;
-            if (in && k > 0 && k < n_out) g = scale * (y[k] + shift - a.labels[at + k]) - gmean;
+            if (in && k > 0 && k < n_out) g = scale * (y[c] + shift - l[c]) - gmean;
             if (in && k < a.ld_dyb) a.dYb[(long long)row * a.ld_dyb + k] = __float2bfloat16_rn(g);
             red[warp][32 * c + lane] = g;
         }
         __syncthreads();
         const int k = k1 + (int)threadIdx.x;
-        if ((int)threadIdx.x < 32 * C && k < n_out) {
+        if ((int)threadIdx.x < CW && k < n_out) {
             float t = 0.f;
 #pragma unroll
             for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
             a.col_part[(long long)blockIdx.x * n_out + k] = t;
         }
         __syncthreads();
+    };
+#pragma unroll
+    for (int h = 0; h < KEEP; ++h)
+        if (h * CW < a.ld_dyb) gradient(h * CW, yk[h], lk[h]);
+    for (int k1 = KEEP * CW; k1 < a.ld_dyb; k1 += CW) {
+        float y[C], l[C];
+        kept_outputs(k1 + lane, y);
+        labels(k1 + lane, l);
+        gradient(k1, y, l);
     }
     if (threadIdx.x == 0) {
         float t = 0.f;
