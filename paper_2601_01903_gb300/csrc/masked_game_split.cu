@@ -666,11 +666,11 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
     while (t < t_end) {
         wait(&ph_ready, ph_parity);
         if (!ok) {
-            finish_pending();
             if (__syncthreads_or(failed ? 1 : 0)) {
                 failed = true;
                 break;
             }
+            finish_pending();  // (after a barrier: see the end of the walk)
             const long long inst = t >> tile_shift;
             const T f = slow_tile<T>(a, a.x + inst * a.d, a.bg + (long long)bgi * a.d, (t - (inst << tile_shift)) << LOW, smA);
             if (tid < ROWS) emit(f, bgi == 0, bgi == a.n_bg - 1, t);
@@ -881,6 +881,9 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
         pend_f2 = c_f2;
         pend_tile = c_t;
     }
+    // The row sums of the pass before may still be read by a slow warp: a pass is
+    // finished only after a barrier that follows the finish of the one before.
+    __syncthreads();
     if (!failed) finish_pending();
     if (__syncthreads_or(failed ? 1 : 0)) {
         // a wait ran out (bounded): no value of this CTA's tiles is vouched for
