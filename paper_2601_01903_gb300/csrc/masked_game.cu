@@ -15,8 +15,7 @@
 // background rows standing in for the absent features) runs as one launch
 // per background row, each adding f / K to v in ascending row order.
 // This kernel serves what the split-digit path (masked_game_split.cu) does
-// not take: hidden widths above 128, fewer than 7 features, and narrow models
-// in float32.
+// not take: hidden widths above 128, fewer than 7 features, and narrow models.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -132,9 +131,9 @@ __global__ void __launch_bounds__(THREADS) masked_game_kernel(Args a) {
 namespace ttfsi_mg {
 
 // v = mean of f over the background rows (one row: the baseline).  Models of
-// up to 128 x 128 hidden units on at least 7 features take the split-digit
-// path on the tensor cores (masked_game_split.cu), one launch; others one
-// launch of masked_game_kernel per row, added in ascending order.
+// up to 128 x 128 hidden units on at least 7 features, narrow ones aside, take
+// the split-digit path on the tensor cores (masked_game_split.cu), one launch;
+// others one launch of masked_game_kernel per row, added in ascending order.
 static tt_fsi_status masked_game_launch(const tt_fsi_mlp *model, const double *x_dev, const double *bg_dev, int n_bg,
                                         int64_t B, void *v_dev, int out_f32, struct CUstream_st *stream) {
     if (!model || B < 0) return TT_FSI_ERR_INVALID_ARG;
@@ -144,7 +143,7 @@ static tt_fsi_status masked_game_launch(const tt_fsi_mlp *model, const double *x
     if (model->d < 1 || model->d > 30 || model->h1 < 1 || model->h2 < 1 || model->h1 > MAX_H || model->h2 > MAX_H)
         return TT_FSI_ERR_INVALID_ARG;
     if (out_f32 && (!model->W2f || !model->b2f || !model->W3f)) return TT_FSI_ERR_INVALID_ARG;
-    if (ttfsi_mgs::split_serves(model->d, model->h1, model->h2, out_f32))
+    if (ttfsi_mgs::split_serves(model->d, model->h1, model->h2, B, out_f32))
         return ttfsi_mgs::split_launch(model, x_dev, bg_dev, n_bg, B, v_dev, out_f32, stream);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     const int g = model->d < G ? model->d : G;

@@ -9,21 +9,53 @@
 // GELUs come next.  Here
 //
 //   layer 2 is a product of integers: the activations of a tile and W2 are cut
-//     to fixed point against a power-of-two scale and written as balanced
-//     base-256 digits (float64: 7 digits = 56 bits, float32: 4 = 32 bits), each
-//     an exact FP16 number.  A product of two digit matrices over K <= 128 has
-//     sums below 2^21, so all products of one diagonal i + j = const add up
-//     exactly in one FP32 accumulator (at most 7 of them, below 2^24): the
-//     Ozaki splitting (Ozaki, Ogita, Oishi & Rump, "Error-free transformations
-//     of matrix multiplication", 2012) with fixed digits.  Diagonals 0 .. 7
-//     (float64, 34 products) or 0 .. 3 (float32, 10) are kept: what is dropped
-//     is below the rounding of the last digit.  The diagonals are put together
-//     in 64-bit integers (float64) or by three fused multiply-adds (float32).
+//     to fixed point and written as balanced base-256 digits (float64: 7 digits =
+//     56 bits, float32: 4 = 32 bits), each an exact FP16 number.  A product of two
+//     digit matrices over K <= 128 has sums below 2^21, so all products of one
+//     diagonal i + j = const add up exactly in one FP32 accumulator (at most 7 of
+//     them, below 2^24): the Ozaki splitting (Ozaki, Ogita, Oishi & Rump,
+//     "Error-free transformations of matrix multiplication", 2012) with fixed
+//     digits.  Diagonals 0 .. 7 (float64, 34 products) or 0 .. 3 (float32, 10) are
+//     kept: what is dropped is below the rounding of the last digit.  The
+//     diagonals are put together in 64-bit integers (float64) or by three fused
+//     multiply-adds (float32).
 //   float64 everywhere else is 64-bit fixed point on the integer pipes, which
 //     are some 60 times as wide as the float64 pipe of this part: layer-1
 //     pre-activations are sums of integers (exact, by subset sums), GELU is
 //     max(z, 0) - |z| Phi(-|z|) with the second term from a table of quintic
 //     polynomials, layer 3 exact 32 x 32-bit products.
+//
+// Scales (all powers of two, so that none of them rounds anything):
+//   a unit of layer 1 has an exponent E, from a bound of its pre-activations over
+//     the instance's coalitions; its activations count in units of 2^E and its
+//     column of W2 is multiplied by 2^E;
+//   a row of W2 (so scaled) has an exponent of its own, undone where the
+//     accumulators are drained, and in float64 a unit of layer 2 a format of its
+//     own (62 bits from its bound down), undone in W3;
+//   a coalition has an exponent e <= 0, from what its features and b1 can give any
+//     unit, undone with the row's: coalitions of small features keep their digits.
+// The model's own exponents, for features of size 2, serve the instances whose
+// bounds they hold, so that one set of W2's slices serves many; an instance
+// beyond them gets its own.
+// The fixed point is taken where what it adds stays below the rounding of the
+// type's own arithmetic:
+//   the digits of a row of W2 end 2^-57 (2^-33) below its largest entry, a double
+//     (float) loses 2^-54 (2^-25) of each product and about sqrt(terms) times that
+//     in their sum: the largest entry may be up to EVEN max(12, 3 sqrt(terms)) times
+//     the mean of the others', weighted by their bounds and averaged over the rows
+//     by |W3|;
+//   the GELU table is off by 2^-59 whatever the result, so in float64 no unit of
+//     layer 2 may carry most of W3 (mu >= 8), W3 has to be even in the same sense
+//     as W2, and a coalition may lie 2^-6 at most below the largest (row_span: less
+//     for units of small pre-activations or an uneven W3); float32's pre-
+//     activations go through floats, and its coalitions may lie 2^-34 below;
+//   one feature may leave the others 2^-8 (float64) or 2^-34 of a unit's bound.
+// A unit that no coalition can lift to -9 is left out (its GELU is 0).  Coalitions
+// below row_span (slow_rows), and instances that the rules refuse, among them all
+// with non-finite values (slow_tiles), are evaluated in the arithmetic of the type.
+// (One exponent for all units of a layer, as this path had at first, lost the bits
+// by which a unit, a bias or a coalition was smaller than the largest: 5e-2 of the
+// values in float32 for one unit 2^28 above the others.)
 //
 // One CTA (16 warps) per SM walks a contiguous range of 128-coalition tiles:
 // layer 1 of a tile into the digit slices in shared memory, one thread issues
@@ -31,17 +63,18 @@
 // before, whose accumulators they drained into registers.
 //
 // Measured on one GB300: float64, 64 instances of a 14-64-64-1 model (2^20
-// coalitions) 19.67 ms on masked_game_kernel, 0.79 ms here; float32, 8
-// instances of a 16-128-128-1 model (2^19) 2.38 ms, 0.255 ms here.  Errors
-// against 120-bit arithmetic are below masked_game_kernel's (relative 2-norms
-// 0.7 to 3e-16 against 0.9 to 5e-16, and 1.1 to 1.9e-7 against 1 to 2.5e-7).
-// Bound: instruction issue of the GELUs (float64: 112 instructions per hidden
-// unit and coalition, 45 % issue; the tensor cores are 14 % busy).
-//
-// Instances (or background rows) whose scale the fixed point does not serve --
-// non-finite values, one feature outweighing all others 256 to 1, in float64
-// pre-activations that all stay below 1/4 or pass 2^16 -- are evaluated by
-// slow_tile in the arithmetic of the type, tile by tile.
+// coalitions) 19.67 ms on masked_game_kernel, 0.80 ms here; float32, 8
+// instances of a 16-128-128-1 model (2^19) 2.38 ms, 0.26 ms here.  Largest
+// errors, coalition by coalition and against extended precision, are 0.3 to 0.9
+// of masked_game_kernel's on even models and at most 1.7 times them over units,
+// biases and features of other scales (2^-28 to 2^28, -1e8, 1e12).  An
+// instance's scales take 1.7 us where the model's serve, 6 us where not, and the
+// model's 6 us at the start.  Instances that are all refused take 0.4 to 0.5 of
+// masked_game_kernel's time in float64; in float32 0.6 (128 x 128 units) to 1.2 (64 x
+// 64, many tiles: 16 warps per SM hide less of the latencies than its 52), 0.4 to 0.5
+// for few tiles.
+// What bounds the fast path is the work of the GELUs at one CTA per SM (its
+// accumulators take the tensor memory, its slices and table the shared memory).
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -79,6 +112,12 @@ struct Cfg {
     static constexpr int NW = F64 ? 64 : 128;  // layer-2 units per pass; ND * NW = 512 TMEM columns
     static constexpr int BITS = F64 ? 55 : 31; // fraction bits of the digit format
     static constexpr int CPT = NW / 4;         // accumulator columns per thread in the epilogue
+    // what the fixed point serves (see above)
+    static constexpr int EMIN = F64 ? 0 : -60, EMAX = F64 ? 19 : 60;  // exponents of a unit of layer 1
+    static constexpr int SPAN = F64 ? 6 : 34;                         // bits between the largest row and a row
+    static constexpr float LONE = F64 ? 0x1p-8f : 0x1p-34f;           // one feature against a unit's others
+    static constexpr float TYPICAL = 2.f;                            // size of a feature that the model's scales allow for
+    static constexpr float EVEN = F64 ? 1.5f : 4.f;                   // digits of W2 below the type's own
 };
 
 // ---- GELU in fixed point ---------------------------------------------------
@@ -88,7 +127,7 @@ struct Cfg {
 // Chebyshev terms are dropped, coefficients rounded to fixed point from the
 // highest down: c0 (62 fraction bits), c1 (71), c2 (80; its low 16 bits hold
 // c5), c3 (57), c4 (58), c5 (59).  Largest error against 160-bit arithmetic
-// 2^-56.9, root mean square 2^-59.4 (float64's own rounding of a result near
+// 2^-56.9, root mean square 2^-59.2 (float64's own rounding of a result near
 // 1/3 is up to 2^-55).
 constexpr int TAB_INTERVALS = 1120;
 constexpr int TAB_ROWS = TAB_INTERVALS + 1;
@@ -122,17 +161,17 @@ __device__ __forceinline__ i64 mul_hi_add(int a_hi, int a_half, i64 b, i64 c, in
     return mad_wide(a_hi, hi32(b), mad_wide(mid, two, c));
 }
 
-// GELU of z = Z 2^-f as an integer of the same format, 43 <= f <= 62.  What
+// GELU of z = Z 2^(s - 62) as an integer of the same format, 0 <= s <= 19.  What
 // bounds it is the integer ALU (half the issue rate), so shifts and adds are
 // left to multiplications where the formats allow it.
-__device__ __forceinline__ i64 gelu_fixed(i64 Z, int f, const ulonglong2 *tab, int two) {
+__device__ __forceinline__ i64 gelu_fixed(i64 Z, int s, const ulonglong2 *tab, int two) {
     const int sign = hi32(Z) >> 31;
     const i64 m = (Z ^ join((unsigned)sign, sign)) - (i64)sign;
     const unsigned mh = (unsigned)hi32(m);
-    const unsigned idx = min(mh >> (f - 39), (unsigned)TAB_INTERVALS);
+    const unsigned idx = min(mh >> (23 - s), (unsigned)TAB_INTERVALS);
     // tau 2^63: the bits below the index, about the centre
-    const int t = (int)(__funnelshift_l(lo32(m), mh, 71 - f) ^ 0x80000000u);
-    const unsigned tlow = lo32(m) << (71 - f);
+    const int t = (int)(__funnelshift_l(lo32(m), mh, 9 + s) ^ 0x80000000u);
+    const unsigned tlow = lo32(m) << (9 + s);
     const ulonglong2 r0 = tab[2 * idx], r1 = tab[2 * idx + 1];
     const int u4 = (int)(r1.y >> 32) + __mulhi(t, (int)(short)(r1.x & 0xffff));
     const int u3 = (int)(unsigned)r1.y + __mulhi(t, u4);
@@ -140,7 +179,7 @@ __device__ __forceinline__ i64 gelu_fixed(i64 Z, int f, const ulonglong2 *tab, i
     const i64 u2 = mad_wide(th, u3, mad_wide(__mulhi(tl, u3), two, (i64)r1.x));
     const i64 u1 = mul_hi_add(th, tl, u2, (i64)r0.y, two);
     const i64 h = mul_hi_add(th, tl, u1, (i64)r0.x, two);  // near z = 0 possibly a unit below 0
-    return (Z & ~join((unsigned)sign, sign)) - shr(h, 62 - f);
+    return (Z & ~join((unsigned)sign, sign)) - shr(h, s);
 }
 
 // GELU in float32 without branches: max(z, 0) - t Phi(-t), t = |z|, with
@@ -183,6 +222,15 @@ __device__ __forceinline__ i64 fix(double v, int f) {
 __device__ __forceinline__ int exp_above(float v) {
     const int e = (int)((__float_as_uint(v) >> 23) & 0xff);
     return e == 0 ? -127 : e - 126;
+}
+
+// |v| cut to a float without float64 arithmetic: 0 below 2^-126, infinite from
+// 2^127 on and for NaN.
+__device__ __forceinline__ float magnitude(double v) {
+    const u64 b = (u64)__double_as_longlong(v);
+    const unsigned hi = (unsigned)(b >> 32) & 0x7fffffffu, e = hi >> 20;
+    const unsigned f = ((e - 896) << 23) | ((hi & 0xfffffu) << 3) | ((unsigned)b >> 29);
+    return __uint_as_float(e < 1023 - 126 ? 0u : e > 1023 + 126 ? 0x7f800000u : f);
 }
 
 // 2^e as a float, -126 <= e <= 127.
@@ -244,6 +292,7 @@ struct Args {
     const double *x, *bg;
     void *v;
     int n_bg, d, h1, h2;
+    int halves;  // 1: two CTAs per tile, each for 64 of its coalitions
     long long n_tiles;
     double scale;
     // powers of two that the compiler must not see through: it would turn the
@@ -255,31 +304,55 @@ struct Args {
 template <bool F64>
 struct Smem {
     using C = Cfg<F64>;
+    static constexpr int CHUNKS = F64 ? 1 : 2;  // K chunks whose tables and W2 slices are kept (float32: all)
     static constexpr int A = 0;
     static constexpr int W = A + C::NS * SLICE_A;
-    static constexpr int W_CHUNKS = F64 ? 1 : 2;  // K chunks of W2 held (float32: all of it)
-    static constexpr int TAB = W + W_CHUNKS * C::NS * C::NW * 128;
+    static constexpr int TAB = W + CHUNKS * C::NS * C::NW * 128;
     static constexpr int PH = TAB + (F64 ? TAB_ROWS * 32 : 0);  // [16][KC] pre-activations by bits 3 .. 6
-    static constexpr int DL = PH + 16 * KC * 8;                 // [7][KC] i64, or two chunks of [7][KC] int
-    static constexpr int PART = DL + LOW * KC * 8;              // [3][ROWS] row sums of column groups 1 .. 3
-    static constexpr int N8A = PART + 3 * ROWS * (F64 ? 16 : 4);              // [NW] 8 bytes: b2 in fixed point | b2, W3
-    static constexpr int N8B = N8A + C::NW * 8;                 // [NW] int2: W3 in fixed point, high and low part
-    static constexpr int L1 = N8B + C::NW * 8;                  // [MAXH] float: row sums of |W2|
-    static constexpr int END = L1 + MAXH * 4;
+    static constexpr int DL = PH + 16 * KC * (F64 ? 8 : 4);     // [CHUNKS][7][KC] i64: a low feature joins
+    static constexpr int DF = DL + CHUNKS * LOW * KC * 8;       // float32: [CHUNKS][3][KC], the first three as floats
+    static constexpr int PART = DF + (F64 ? 0 : CHUNKS * 3 * KC * 4);  // [3][ROWS] row sums of column groups 1 .. 3
+    static constexpr int COL = PART + 3 * ROWS * (F64 ? 16 : 4);  // [NW] 16 bytes: b2 and W3 in fixed point | b2, W3, 2^ew
+    static constexpr int CS = COL + C::NW * 16;                 // float64: [NW] 62 - f
+    static constexpr int CE = CS + (F64 ? C::NW * 4 : 0);       // float64: [NW] ew + f - 38
+    static constexpr int SE = CE + (F64 ? C::NW * 4 : 0);       // [MAXH] exponent of a unit of layer 1 + 64, kDead
+    static constexpr int EW = SE + MAXH * 4;                    // [MAXH] exponent of a row of W2, or kDead
+    static constexpr int FN = EW + MAXH * 4;                    // float64: [MAXH] fraction bits of a unit of layer 2
+    static constexpr int ER = FN + (F64 ? MAXH * 4 : 0);        // [2][ROWS] exponents of the rows, double-buffered
+    static constexpr int MW = ER + 2 * ROWS * 4;                // [32] float: a feature's largest scaled weight, b1's
+    static constexpr int MB = MW + 32 * 4;                      // [32] float: a feature's largest background value
+    static constexpr int END = MB + 32 * 4;
     static constexpr int BYTES = END + 1024;
 };
 static_assert(Smem<true>::BYTES <= 232448 - 1024 && Smem<false>::BYTES <= 232448 - 1024, "fits one CTA per SM");
+constexpr int kDead = 1 << 10;
 
-// Largest (op > 0) or smallest value over the CTA; every thread gets it.
-__device__ __forceinline__ int block_max(int v, int *red) {
-    v = __reduce_max_sync(0xffffffffu, v);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    int m = red[0];
+// N values over the CTA, the first NSUM of them summed (in a fixed order), the
+// rest maximised (none of them negative); every thread gets them.
+template <int N, int NSUM>
+__device__ __forceinline__ void block_reduce(float (&v)[N], float (&red)[WARPS][10]) {
+    static_assert(N <= 10, "red");
 #pragma unroll
-    for (int w = 1; w < WARPS; ++w) m = max(m, red[w]);
-    return m;
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float u = __shfl_xor_sync(0xffffffffu, v[i], o);
+            v[i] = i < NSUM ? v[i] + u : fmaxf(v[i], u);
+        }
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int i = 0; i < N; ++i) red[threadIdx.x >> 5][i] = v[i];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        v[i] = red[threadIdx.x & (WARPS - 1)][i];
+#pragma unroll
+        for (int o = WARPS / 2; o > 0; o >>= 1) {
+            const float u = __shfl_xor_sync(0xffffffffu, v[i], o);
+            v[i] = i < NSUM ? v[i] + u : fmaxf(v[i], u);
+        }
+    }
 }
 
 template <typename T>
@@ -297,54 +370,439 @@ struct Weights<float> {
     static __device__ __forceinline__ const float *w3(const Args &a) { return a.W3f; }
 };
 
-// One tile of one background row in the arithmetic of the type (64 coalitions
-// at a time; eight threads share a coalition's layer 2): thread c < 128
-// returns f of coalition c.
-template <typename T>
-__device__ __noinline__ T slow_tile(const Args &a, const double *x, const double *base, long long S_high,
-                                    unsigned char *smem) {
-    T *pre = reinterpret_cast<T *>(smem);
-    T *part = pre + 64 * (MAXH + 1);
-    const int tid = threadIdx.x, ld = a.h1 + 1;
-    T result = 0;
-    for (int half = 0; half < 2; ++half) {
-        const long long S0 = S_high | (half << 6);
-        for (int j = tid; j < a.h1; j += THREADS) {
-            double acc = a.b1[j];
-            for (int i = 0; i < a.d; ++i) {
-                const bool on = i >= 6 && ((S0 >> i) & 1);
-                acc += a.W1[(long long)j * a.d + i] * (on ? x[i] : base[i]);
-            }
-            pre[j] = (T)acc;
-            for (int k = 0; k < 6; ++k) {
-                const T delta = (T)(a.W1[(long long)j * a.d + k] * (x[k] - base[k]));
-                for (int c = 0; c < (1 << k); ++c) pre[(c | (1 << k)) * ld + j] = pre[c * ld + j] + delta;
-            }
-        }
-        __syncthreads();
-        for (int idx = tid; idx < 64 * a.h1; idx += THREADS) {
-            const int c = idx / a.h1, j = idx - c * a.h1;
-            pre[c * ld + j] = gelu_of(pre[c * ld + j]);
-        }
-        __syncthreads();
-        const int c = tid & 63, q = tid >> 6;
-        T acc3 = 0;
-        for (int n = q; n < a.h2; n += 8) {
-            T acc = Weights<T>::b2(a)[n];
-            const T *w = Weights<T>::w2(a) + (long long)n * a.h1;
-            for (int i = 0; i < a.h1; ++i) acc += __ldg(w + i) * pre[c * ld + i];
-            acc3 += Weights<T>::w3(a)[n] * gelu_of(acc);
-        }
-        part[tid] = acc3;
-        __syncthreads();
-        if ((tid >> 6) == half) {
-            T s = part[c];
-            for (int k = 1; k < 8; ++k) s += part[c + 64 * k];
-            result = s + (T)a.b3;
-        }
-        __syncthreads();
+// GELU of the rows below: erff, and in float64 (whose pipe bounds them) the table
+// where its 2^-59 is below the rounding of the result: for 2^-4 <= |z| < 8, z
+// an exact multiple of 2^-58; below, z Phi(z) = z / 2 + z^2 (1 - z^2 / 6 + z^4 / 40 -
+// ...) / sqrt(2 pi), Taylor's series of Phi.
+__device__ __forceinline__ float gelu_slow(float z, const ulonglong2 *, int) { return gelu_of(z); }
+__device__ __forceinline__ double gelu_slow(double z, const ulonglong2 *tab, int two) {
+    const float m = magnitude(z);
+    if (m >= 0.0625f && m < 8.f) {
+        const int s = m < 1.f ? 1 : 4;
+        return (double)gelu_fixed(fix(z, 62 - s), s, tab, two) * (m < 1.f ? 0x1p-61 : 0x1p-58);
     }
+    if (m < 0.0625f) {
+        const double y = z * z;
+        double p = fma(y, 1.0 / 599040, -1.0 / 42240);
+        p = fma(y, p, 1.0 / 3456);
+        p = fma(y, p, -1.0 / 336);
+        p = fma(y, p, 1.0 / 40);
+        p = fma(y, p, -1.0 / 6);
+        p = fma(y, p, 1.0);
+        return fma(y * 0.39894228040143267794, p, 0.5 * z);
+    }
+    if (m >= 8.75f && m < 1e38f) return z > 0.0 ? z : -0.0;  // (1 + erf is 2 or 0)
+    return gelu_of(z);
+}
+
+// Layer 2 (GELU) and layer 3 of one coalition for units n0, n0 + step, ...,
+// NB neighbours at a time.
+template <typename T, int NB>
+__device__ __forceinline__ T slow_units(const Args &a, const T *row, int n0, int step, const ulonglong2 *tab) {
+    const T *w2 = Weights<T>::w2(a), *b2 = Weights<T>::b2(a), *w3 = Weights<T>::w3(a);
+    const bool by_four = sizeof(T) == 4 && a.h1 % 4 == 0 && (reinterpret_cast<uintptr_t>(w2) & 15) == 0;
+    T sum = 0;
+    for (int n = n0; n < a.h2; n += step) {
+        T acc[NB];
+        const T *w[NB];
+#pragma unroll
+        for (int k = 0; k < NB; ++k) {
+            const int m = min(n + k, a.h2 - 1);
+            acc[k] = b2[m];
+            w[k] = w2 + m * a.h1;
+        }
+        int i = 0;
+        if constexpr (sizeof(T) == 4) {
+            if (by_four) {
+#pragma unroll 2
+                for (; i < a.h1; i += 4) {
+#pragma unroll
+                    for (int k = 0; k < NB; ++k) {
+                        const float4 v = __ldg(reinterpret_cast<const float4 *>(w[k] + i));
+                        acc[k] += v.x * row[i];
+                        acc[k] += v.y * row[i + 1];
+                        acc[k] += v.z * row[i + 2];
+                        acc[k] += v.w * row[i + 3];
+                    }
+                }
+            }
+        }
+#pragma unroll 8
+        for (; i < a.h1; ++i) {
+            const T r = row[i];
+#pragma unroll
+            for (int k = 0; k < NB; ++k) acc[k] += __ldg(w[k] + i) * r;
+        }
+#pragma unroll
+        for (int k = 0; k < NB; ++k)
+            if (n + k < a.h2) sum += w3[n + k] * gelu_slow(acc[k], tab, a.two);
+    }
+    return sum;
+}
+
+// Shared memory of a team for 64 coalitions, in elements of the type:
+// pre-activations [64][h1 + 1], those without the six low bits, what each of
+// these adds, sums, values, and the list of rows.
+constexpr int SLOW_FEW = 8;  // rows up to which a unit's products are split over lanes
+__host__ __device__ constexpr int slow_elems(int h1) { return 64 * (h1 + 1) + 7 * h1 + SLOW_FEW * MAXH + 64 + 16; }
+static_assert(2 * slow_elems(MAXH) * 8 <= Smem<true>::TAB && 4 * slow_elems(MAXH) * 4 <= Smem<false>::TAB,
+              "two or four teams fit");
+template <typename T>
+__device__ __forceinline__ T *slow_values(T *scratch, int h1) { return scratch + 64 * (h1 + 1) + 7 * h1 + SLOW_FEW * MAXH; }
+
+// The rows given (bit c: coalition S0 | c) of the 64 coalitions from S0 on and one
+// background row in the arithmetic of the type, as masked_game_kernel has it, by
+// a team of threads with a named barrier of its own: slow_values(scratch)[k] = f
+// of the k-th of the rows.
+template <typename T>
+__device__ __forceinline__ void slow_group(const Args &a, const double *x, const double *base, int S0,
+                                           unsigned long long rows, T *scratch, int tid, int team, int barrier,
+                                           const ulonglong2 *tab) {
+    const int warp = tid >> 5, lane = tid & 31, ld = a.h1 + 1, q = tid & 3;
+    T *const pre = scratch, *const high = pre + 64 * ld, *const delta = high + a.h1, *const part = delta + 6 * a.h1;
+    T *const value = slow_values(scratch, a.h1);
+    unsigned char *const list = reinterpret_cast<unsigned char *>(value + 64);
+    auto team_sync = [&] {
+        __syncwarp();
+        asm volatile("barrier.sync %0, %1;" ::"r"(barrier), "r"(team) : "memory");
+    };
+    const int n_rows = __popcll(rows);
+    if (tid < 64 && ((rows >> tid) & 1)) list[__popcll(rows & ((1ull << tid) - 1))] = (unsigned char)tid;
+    for (int j0 = 0; j0 < a.h1; j0 += team / 4) {
+        const int j = j0 + (tid >> 2);
+        double acc = 0.0;
+        if (j < a.h1) {
+            const double *w1 = a.W1 + j * a.d;
+#pragma unroll 4
+            for (int i = q; i < a.d; i += 4) acc += w1[i] * (i >= 6 && ((S0 >> i) & 1) ? x[i] : base[i]);
+            for (int k = q; k < 6; k += 4) delta[k * a.h1 + j] = (T)(w1[k] * (x[k] - base[k]));
+        }
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+        if (q == 0 && j < a.h1) high[j] = (T)(a.b1[j] + acc);
+    }
+    team_sync();
+    const int rows_on = team / a.h1, units_on = team - rows_on * a.h1;
+    for (int c = tid / a.h1, j = tid - c * a.h1; c < n_rows;) {
+        const int bits = list[c];
+        T z = high[j];
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+            if ((bits >> k) & 1) z += delta[k * a.h1 + j];
+        pre[c * ld + j] = gelu_slow(z, tab, a.two);
+        c += rows_on;
+        j += units_on;
+        if (j >= a.h1) {
+            j -= a.h1;
+            ++c;
+        }
+    }
+    team_sync();
+    int groups;
+    if (n_rows <= SLOW_FEW) {
+        // eight lanes share the products of a unit of layer 2
+        groups = a.h2;
+        const T *w2 = Weights<T>::w2(a), *b2 = Weights<T>::b2(a), *w3 = Weights<T>::w3(a);
+        const int items = n_rows * a.h2;
+        for (int i0 = 0; i0 < items; i0 += team / 8) {
+            const int item = i0 + (tid >> 3), n = item / n_rows, c = item - n * n_rows;
+            T acc = 0;
+            if (item < items) {
+#pragma unroll 4
+                for (int i = tid & 7; i < a.h1; i += 8) acc += __ldg(w2 + n * a.h1 + i) * pre[c * ld + i];
+            }
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (item < items && (tid & 7) == 0) part[item] = acc;
+        }
+        team_sync();
+        for (int item = tid; item < items; item += team) {
+            const int n = item / n_rows;
+            part[item] = w3[n] * gelu_slow(b2[n] + part[item], tab, a.two);
+        }
+    } else {
+        // thread (coalition c, group g of units)
+        groups = team / n_rows;
+        const int c = tid % n_rows, g = tid / n_rows;
+        if (g < groups)
+            part[tid] = a.h2 >= 8 * groups ? slow_units<T, 4>(a, pre + c * ld, 4 * g, 4 * groups, tab)
+                                           : slow_units<T, 1>(a, pre + c * ld, g, groups, tab);
+    }
+    team_sync();
+    for (int k = warp; k < n_rows; k += team / 32) {
+        T sum = 0;
+        for (int g = lane; g < groups; g += 32) sum += part[g * n_rows + k];
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (lane == 0) value[k] = sum + (T)a.b3;
+    }
+    team_sync();
+}
+
+// Listed rows of one tile and background row (bit r of the mask: row r): thread
+// r < 128 returns f of row r.  Each half of the CTA takes 64 rows.
+template <typename T>
+__device__ __noinline__ T slow_rows(const Args &a, int tile, int bgi, uint4 mask, unsigned char *smem) {
+    T *const scratch = reinterpret_cast<T *>(smem);
+    const ulonglong2 *tab = reinterpret_cast<const ulonglong2 *>(smem + Smem<true>::TAB);  // (float64)
+    const int tile_shift = a.d - LOW, inst = tile >> tile_shift, S = (tile - (inst << tile_shift)) << LOW;
+    const unsigned long long low = ((unsigned long long)mask.y << 32) | mask.x, high = ((unsigned long long)mask.w << 32) | mask.z;
+    const int half = threadIdx.x / (THREADS / 2);
+    if (half ? high : low)
+        slow_group<T>(a, a.x + (long long)inst * a.d, a.bg + (long long)bgi * a.d, S | (half << 6), half ? high : low,
+                      scratch + half * slow_elems(a.h1), threadIdx.x % (THREADS / 2), THREADS / 2, 1 + half, tab);
+    __syncthreads();
+    T result = 0;
+    if (threadIdx.x < ROWS) {
+        const int r = threadIdx.x & 63, h = threadIdx.x >> 6;
+        const unsigned long long m = h ? high : low;
+        if ((m >> r) & 1) result = slow_values(scratch + h * slow_elems(a.h1), a.h1)[__popcll(m & ((1ull << r) - 1))];
+    }
+    __syncthreads();
     return result;
+}
+
+// All values of tiles [t0, t1) of one instance (halves: of 64 coalitions of the
+// one tile t0): teams of 128, 256 or 512 threads take 64 coalitions at a time, as
+// the CTAs of masked_game_kernel do, each at its own pace.
+template <typename T>
+__device__ __noinline__ void slow_tiles(const Args &a, int t0, int t1, unsigned char *smem) {
+    constexpr int BYTES = Smem<sizeof(T) == 8>::TAB;  // the activations' and W2's regions
+    const int first = a.halves ? 2 * t0 + ((int)blockIdx.x & 1) : 2 * t0, end = a.halves ? first + 1 : 2 * t1;
+    int teams = end - first >= 4 ? 4 : end - first;  // (1, 2 or 4: a tile has two halves)
+    if (teams * slow_elems(a.h1) * (int)sizeof(T) > BYTES) teams = 2;
+    const int team = THREADS / teams, k = threadIdx.x / team, tid = threadIdx.x - k * team;
+    T *const scratch = reinterpret_cast<T *>(smem) + k * slow_elems(a.h1);
+    const ulonglong2 *tab = reinterpret_cast<const ulonglong2 *>(smem + Smem<true>::TAB);  // (float64)
+    const int tile_shift = a.d - LOW, inst = t0 >> tile_shift;
+    const double *x = a.x + (long long)inst * a.d;
+    for (int h = first + k; h < end; h += teams) {
+        T sum = 0;
+        for (int b = 0; b < a.n_bg; ++b) {
+            slow_group<T>(a, x, a.bg + (long long)b * a.d, (h - (inst << (tile_shift + 1))) << 6, ~0ull, scratch, tid, team,
+                          1 + k, tab);
+            if (tid < 64) {
+                const T f = slow_values(scratch, a.h1)[tid];
+                sum = a.n_bg == 1 ? f : b == 0 ? (T)a.scale * f : sum + (T)a.scale * f;
+            }
+        }
+        if (tid < 64) reinterpret_cast<T *>(a.v)[(long long)h * 64 + tid] = sum;
+    }
+    __syncthreads();
+}
+
+// The scales in place, besides the arrays in Smem.
+struct Scales {
+    int ok;        // the instance's rows may take the fixed point
+    int version;   // of the arrays
+    int row_span;  // rows down to 2^-row_span of the largest do
+    int xmax, Q;   // float64: the most extra bits of a row in layer 2; fraction bits of layer 3 less a unit's
+    int model_now, model_ok;         // the model's own scales are in place; they are of use
+    float model_room;                // rounding of the type over what the digits add, at the model's bounds
+    float model_al;                  // sum of those bounds in units of 2^E
+    int const_x, const_Q;            // xmax and Q of the per-unit constants in place
+    signed char model_e[MAXH];       // the model's exponents (127: a unit without weights)
+    float redf[WARPS][10];
+};
+
+// Bounds of unit tid >> 2 over an instance's coalitions (x = null: for features
+// of size C::TYPICAL): |z| <= beta, z <= zmax; lone: one feature leaves less to
+// the others than the format spares.  Also the unit's |W1| (feature q + 4 k) and |b1|.
+template <bool F64>
+__device__ __forceinline__ void unit_bounds(const Args &a, const double *x, const float *most, float &beta, float &zmax,
+                                            bool &lone, float (&w1)[8], float &b) {
+    using C = Cfg<F64>;
+    const int j = threadIdx.x >> 2, q = threadIdx.x & 3;
+    const bool in = j < a.h1;
+    float m[8];
+    const double bias = in ? a.b1[j] : 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {  // (d <= 30; all loads in flight)
+        const int i = q + 4 * k;
+        const bool on = in && i < a.d;
+        w1[k] = on ? magnitude(a.W1[(long long)j * a.d + i]) : 0.f;
+        m[k] = !on ? 0.f : x ? fmaxf(magnitude(x[i]), most[i]) : C::TYPICAL;
+    }
+    float sum = 0.f, top = 0.f, rest = 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const float c = w1[k] * m[k];
+        sum += c;  // (infinite or NaN if anything is)
+        rest += fminf(c, top);
+        top = fmaxf(top, c);
+    }
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+        const float t2 = __shfl_xor_sync(0xffffffffu, top, o);
+        rest += __shfl_xor_sync(0xffffffffu, rest, o) + fminf(top, t2);
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        top = fmaxf(top, t2);
+    }
+    b = magnitude(bias);
+    beta = sum + b;
+    zmax = bias < 0.0 ? sum - b : sum + b;
+    rest += b;
+    lone = rest > 0.f && rest < C::LONE * top;
+}
+
+// Scales for an instance, or the model's own (x = null): exponents of the
+// units of layer 1 and of the rows of W2 (scaled by its columns' exponents),
+// formats of layers 2 and 3, and whether what the digits add stays below the
+// type's own rounding (see the head of the file).  The whole CTA calls it.
+template <bool F64>
+__device__ __noinline__ void set_scales(const Args &a, const double *x, unsigned char *sm, Scales &sc) {
+    using C = Cfg<F64>;
+    using S = Smem<F64>;
+    int *sE = reinterpret_cast<int *>(sm + S::SE), *sEw = reinterpret_cast<int *>(sm + S::EW);
+    int *sFn = reinterpret_cast<int *>(sm + S::FN), *sMW = reinterpret_cast<int *>(sm + S::MW);
+    float *sAl = reinterpret_cast<float *>(sm + S::PART);
+    const int tid = threadIdx.x, lane = tid & 31, n = tid >> 2, q = tid & 3;
+    float beta, zmax, w1[8], b1;
+    bool lone;
+    if (x) {
+        // the model's scales serve where they hold the bounds with room to
+        // spare, so that one set of W2's slices serves many instances
+        unit_bounds<F64>(a, x, reinterpret_cast<const float *>(sm + S::MB), beta, zmax, lone, w1, b1);
+        const bool bad = !(beta < 1e20f), dead = !(beta > 0.f) || zmax < -9.f;
+        const float b = sc.model_e[n] == 127 ? 0.f : beta * pow2(-sc.model_e[n]);
+        // (a unit's bound is in four threads); 1: not in the model's scales, 2: refused
+        float v[2] = {bad || dead ? 0.f : 0.25f * b, bad || (lone && !dead) ? 2.f : 1.01f * b >= 1.f ? 1.f : 0.f};
+        block_reduce<2, 1>(v, sc.redf);
+        const bool refused = v[1] == 2.f;
+        const bool fits = v[1] == 0.f && sc.model_ok && v[0] * sc.model_room >= sc.model_al;
+        if (refused || (fits && sc.model_now)) {
+            if (tid == 0) sc.ok = !refused;
+            __syncthreads();
+            return;
+        }
+        if (fits) x = nullptr;  // back to the model's
+    }
+    const bool model = !x;
+    if (model) {
+        unit_bounds<F64>(a, nullptr, nullptr, beta, zmax, lone, w1, b1);
+        if (zmax < -9.f) zmax = 0.f;  // dead for some instances only
+    }
+    if (tid < 32) sMW[tid] = 0;
+
+    bool bad = !(beta < 1e20f);
+    const bool dead = !(beta > 0.f) || zmax < -9.f;  // no activation that counts
+    const int e = max(dead || bad ? C::EMIN : exp_above(1.01f * beta), C::EMIN);
+    bad |= e > C::EMAX;
+    const float al = dead || bad ? 0.f : beta * pow2(-e);
+    if (q == 0) {
+        sE[n] = (min(e, C::EMAX) + 64) | (dead ? kDead : 0);
+        sAl[n] = al;
+        if (sc.version == 0) sc.model_e[n] = dead ? 127 : (signed char)min(e, C::EMAX);
+    }
+    __syncthreads();
+    // a feature's (at d: b1's) largest weight in units of 2^E
+    const float unit = dead || bad ? 0.f : pow2(-e);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        float m = w1[k] * unit;
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (lane < 4 && q + 4 * k < a.d) atomicMax(sMW + q + 4 * k, __float_as_int(m));  // none is negative
+    }
+    const int b_most = __reduce_max_sync(0xffffffffu, __float_as_int(b1 * unit));
+    if (lane == 0) atomicMax(sMW + a.d, b_most);
+
+    float wmax = 0.f, wsum = 0.f, nat = 0.f, top = 0.f;
+    int count = 0;
+    double bias2 = 0.0, weight3 = 0.0;
+    if (n < a.h2) {
+        bias2 = a.b2[n];
+        weight3 = a.W3[n];
+#pragma unroll 8
+        for (int j = q; j < a.h1; j += 4) {
+            const float m = magnitude(a.W2[(long long)n * a.h1 + j]);
+            bad |= !(m < 1e20f);
+            const float w = (sE[j] & kDead) ? 0.f : m * pow2((sE[j] & 255) - 64), c = w * sAl[j];
+            wmax = fmaxf(wmax, w);
+            wsum += w;
+            nat += c;
+            top = fmaxf(top, c);
+            count += c > 0.f;
+        }
+    }
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+        wmax = fmaxf(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
+        top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+        wsum += __shfl_xor_sync(0xffffffffu, wsum, o);
+        nat += __shfl_xor_sync(0xffffffffu, nat, o);
+        count += __shfl_xor_sync(0xffffffffu, count, o);
+    }
+    const float b2 = magnitude(bias2), w3 = magnitude(weight3);
+    bad |= !(b2 < 1e20f) || !(w3 < 1e18f) || (weight3 != 0.0 && w3 < 1e-18f) || !(wsum < 1e18f);
+    const float zb = 1.02f * wsum + b2;
+    const bool live = w3 > 0.f && !((bias2 < 0.0 ? 1.02f * wsum - b2 : zb) < -9.f);
+    const int ze = exp_above(zb);
+    int ew = max(exp_above(1.01f * wmax), -60), fn = 0, xmax = 0, x_b2 = 0;
+    if constexpr (F64) {
+        // a row whose activations are 2^-x of the largest keeps x more bits of
+        // layer 2 where b2 allows it and the format, of 62 bits, has them
+        float less[2] = {live && b2 > 0.f ? (float)max(0, C::SPAN - max(0, ze - exp_above(b2))) : 0.f,
+                         live ? (float)max(0, C::SPAN - max(0, 1 + ze)) : 0.f};
+        block_reduce<2, 0>(less, sc.redf);
+        x_b2 = C::SPAN - (int)less[0];
+        xmax = min(x_b2, C::SPAN - (int)less[1]);
+        fn = live ? min(61 - ze, 62 - xmax) : 62 - xmax;
+        ew = max(ew, 45 - fn);
+        bad |= live && ze > 18;
+    } else {
+        bad |= ew > 60;
+    }
+    if (q == 0) {
+        sEw[n] = live ? ew : kDead;
+        if constexpr (F64) sFn[n] = fn;
+    }
+    // the digits of W2 end 2^-57 (float64) or 2^-33 (float32) below the largest of
+    // a row; the type itself loses 2^-54 or 2^-25 of each product and more in sums
+    const bool on = q == 0 && live, several = on && count > 1;
+    const float k_row = C::EVEN * fmaxf(12.f, 3.f * sqrtf((float)count));
+    constexpr int NV = F64 ? 10 : 3, NS = F64 ? 8 : 3;
+    float v[NV];
+    v[0] = several ? w3 * wmax * (float)(count - 1) : 0.f;
+    v[1] = several ? w3 * k_row * (nat - top) : 0.f;
+    v[2] = q == 0 ? al : 0.f;
+    if constexpr (F64) {
+        v[3] = on ? w3 * zb : 0.f;                        // what a unit can give layer 3
+        v[4] = on ? w3 * fminf(1.f, 0.125f * zb) : 0.f;   // and about gives
+        v[5] = on ? w3 * w3 : 0.f;
+        v[6] = on ? 1.f : 0.f;
+        v[7] = q == 0 && !dead ? (float)(e + 4096) : 0.f;  // exponents and (4096 each) number of live units
+        v[8] = on ? w3 * pow2(61 - fn) : 0.f;
+        v[9] = on ? w3 * zb : 0.f;
+    }
+    block_reduce<NV, NS>(v, sc.redf);
+    bool ok = !__syncthreads_or(bad);
+    if (tid == 0) {
+        const float room = v[0] > 0.f ? v[1] / v[0] : 1e30f;
+        sc.row_span = C::SPAN;
+        sc.xmax = sc.Q = 0;
+        if constexpr (F64) {
+            const float units = v[6], live_units = floorf(v[7] * (1.f / 4096.f));
+            if (units > 1.f)  // W3's 53 bits of its largest against the units' own
+                ok = ok && v[8] * (units - 1.f) <= 2.f * fmaxf(12.f, 3.f * sqrtf(units)) * (v[3] - v[9]);
+            // the table's 2^-59 against what double loses of what the units give
+            const float mu = v[5] > 0.f ? 128.f * v[4] * rsqrtf(v[5] * units) : 1e30f;
+            const int e_mean = live_units > 0.f ? (int)floorf((v[7] - 4096.f * live_units) / live_units) : C::SPAN;
+            sc.row_span = min(min(C::SPAN, e_mean + 3), exp_above(mu) - 2);
+            if (xmax < x_b2) sc.row_span = min(sc.row_span, xmax + 1);
+            ok = ok && mu >= 8.f;
+            sc.xmax = xmax;
+            sc.Q = 114 - max(exp_above(v[8]), -60);
+        }
+        if (sc.version == 0) {
+            sc.model_ok = ok;
+            sc.model_room = room;
+            sc.model_al = v[2];
+        }
+        sc.version += 1;
+        sc.model_now = model;
+        sc.ok = ok && (model || room >= 1.f);
+    }
+    __syncthreads();
 }
 
 template <bool F64>
@@ -352,22 +810,27 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
     using C = Cfg<F64>;
     using S = Smem<F64>;
     using T = typename std::conditional<F64, double, float>::type;
-    constexpr int NS = C::NS, ND = C::ND, NW = C::NW, BITS = C::BITS, CPT = C::CPT;
+    constexpr int NS = C::NS, ND = C::ND, NW = C::NW, BITS = C::BITS, CPT = C::CPT, CHUNKS = S::CHUNKS;
     extern __shared__ __align__(1024) unsigned char sm_raw[];
     const uint32_t raw = smem_u32(sm_raw);
     unsigned char *sm = sm_raw + (((raw + 1023) & ~1023u) - raw);
     unsigned char *smA = sm + S::A, *smW = sm + S::W;
     ulonglong2 *tab = reinterpret_cast<ulonglong2 *>(sm + S::TAB);
-    // layer-1 pre-activations: 62 (float64) or 30 (float32) fraction bits of 2^E
-    using P = typename std::conditional<F64, i64, int>::type;
-    constexpr int PBITS = F64 ? 62 : 30;
-    constexpr int CHUNKS = F64 ? 1 : 2;  // K chunks whose tables are kept
+    // layer-1 pre-activations: sums of integers with 62 fraction bits of the
+    // unit's 2^E; float32 takes them up from bits 3 .. 6 on as floats
+    using P = typename std::conditional<F64, i64, float>::type;
     P *PH = reinterpret_cast<P *>(sm + S::PH);
-    P *DL = reinterpret_cast<P *>(sm + S::DL);
-    float *sL1 = reinterpret_cast<float *>(sm + S::L1);
+    i64 *DL = reinterpret_cast<i64 *>(sm + S::DL);
+    float *DF = reinterpret_cast<float *>(sm + S::DF);
+    int *sE = reinterpret_cast<int *>(sm + S::SE), *sEw = reinterpret_cast<int *>(sm + S::EW);
+    int *sFn = reinterpret_cast<int *>(sm + S::FN), *sEr = reinterpret_cast<int *>(sm + S::ER);
+    int *sCs = reinterpret_cast<int *>(sm + S::CS), *sCe = reinterpret_cast<int *>(sm + S::CE);
+    const float *sMW = reinterpret_cast<const float *>(sm + S::MW);
+    int *sMB = reinterpret_cast<int *>(sm + S::MB);
     __shared__ __align__(8) uint64_t mbar, ph_ready, part_ready;  // MMAs done; tables made; row sums written
     __shared__ uint32_t tmem_sh;
-    __shared__ int red[WARPS];
+    __shared__ Scales sc;
+    __shared__ __align__(16) unsigned sFlag[2][4];  // rows left to slow_rows, double-buffered
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
@@ -379,44 +842,30 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_sh)), "r"(512));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+        sMB[lane] = 0;
+        if (lane == 0) sc.version = 0;
     }
     if constexpr (F64)
         for (int i = tid; i < TAB_ROWS * 2; i += THREADS) tab[i] = (&g_gelu_table[0][0])[i];
-
-    // ---- once per CTA: the scale of W2 (2^ew), its row sums, the scale of W3 ----
-    int ew, e3;
-    bool model_ok;
-    float ab2 = 0.f;  // |b2| of unit tid >> 2
-    {
-        const int n = tid >> 2, q = tid & 3;
-        float mx = 0.f, sum = 0.f, aw3 = 0.f;
-        if (n < a.h2) {
-            for (int j = q; j < a.h1; j += 4) {
-                const float w = fabsf((float)a.W2[(long long)n * a.h1 + j]);
-                mx = fmaxf(mx, w);
-                sum += w;  // carries a NaN or an infinity on
-            }
-            ab2 = fabsf((float)a.b2[n]);
-            aw3 = fabsf((float)a.W3[n]);
-        }
-        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-        sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-        if (q == 0) sL1[n] = sum;
-        ew = block_max(exp_above(1.01f * mx), red);
-        e3 = block_max(exp_above(aw3), red);
-        const bool bad = !(sum < 1e20f) || !(ab2 < 1e20f) || !(aw3 < 1e20f);
-        model_ok = block_max(bad ? 1 : 0, red) == 0 && e3 < 60;
-        ew = max(ew, -60);  // an all-zero W2 has any scale
-        e3 = max(e3, -60);
-    }
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_sh;
+    if (lane < a.d) {
+        float m = 0.f;
+        for (int k = warp; k < a.n_bg; k += WARPS) m = fmaxf(m, magnitude(a.bg[(long long)k * a.d + lane]));
+        atomicMax(sMB + lane, __float_as_int(m));  // none is negative
+    }
+    __syncthreads();
     const uint32_t a_base = smem_u32(smA), w_base = smem_u32(smW);  // below 2^18: descriptors add up
 
     const int n_kc = (a.h1 + KC - 1) / KC, n_nh = (a.h2 + NW - 1) / NW;
     const int tile_shift = a.d - LOW;
-    const long long t_begin = a.n_tiles * blockIdx.x / gridDim.x, t_end = a.n_tiles * (blockIdx.x + 1) / gridDim.x;
+    // (2^31 tiles would be 2^38 values)
+    const int t_begin = a.halves ? (int)blockIdx.x >> 1 : (int)(a.n_tiles * blockIdx.x / gridDim.x);
+    const int t_end = a.halves ? t_begin + 1 : (int)(a.n_tiles * (blockIdx.x + 1) / gridDim.x);
+    // the rows this CTA gives out, by quarters
+    auto own = [&](int quarter) { return !a.halves || (quarter >> 1) == (blockIdx.x & 1) ? ~0u : 0u; };
+    const bool own_row = tid < ROWS && own(warp);
     uint32_t parity = 0, ph_parity = 0, part_parity = 0;
     bool failed = false;  // a bounded wait ran out (of this warp until the CTA's barrier)
     // a warp's arrival and wait (lane 0 for the warp, bounded)
@@ -432,6 +881,8 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
         phase ^= 1u;
     };
 
+    set_scales<F64>(a, nullptr, sm, sc);
+
     // epilogue state: the accumulators of the pass in flight, its row sums so
     // far, and (threads < 128) the sum over background rows of row tid
     i64 zi[F64 ? CPT : 1];
@@ -439,37 +890,42 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
     i64 acc_hh = 0, acc_hl = 0, acc_lh = 0, acc_ll = 0;
     float acc_f = 0.f;
     T vsum = 0;
-    bool pending = false, pend_last_nh = false, pend_first_bg = false, pend_last_bg = false;
-    int pend_f2 = 0;
-    long long pend_tile = 0;
+    bool slow = false;  // row tid of the tile and background row came from slow_rows
+    enum : int { kWaiting = 1, kLastPass = 2, kFirstBg = 4, kLastBg = 8, kSlow = 16 };
+    int pend = 0;       // the pass in flight
+    int pend_x = 0, pend_tile = 0;
 
     // epilogue: thread (row, quarter of the pass's columns), in whole loads of 8
     const int n_col = min(NW, a.h2);
     const int cpt = min(CPT, ((n_col + 31) >> 5) << 3);
     const int erow = 32 * (warp & 3) + lane, ecol = (warp >> 2) * cpt;
 
-    auto emit = [&](T f, bool first, bool last, long long tile) {  // threads < 128
+    auto emit = [&](T f, bool first, bool last, int tile) {  // threads < 128
         if (a.n_bg == 1)
             vsum = f;
         else
             vsum = first ? (T)a.scale * f : vsum + (T)a.scale * f;
-        if (last) reinterpret_cast<T *>(a.v)[tile * ROWS + tid] = vsum;
+        if (last && own_row) reinterpret_cast<T *>(a.v)[(long long)tile * ROWS + tid] = vsum;
+    };
+    auto emit_pending = [&](T f) {  // a slow row's value is in already
+        if (!(pend & kSlow)) emit(f, pend & kFirstBg, pend & kLastBg, pend_tile);
     };
 
     // Layers 2 (GELU) and 3 of the drained accumulators.
     auto finish_pending = [&]() {
-        if (!pending) return;
-        pending = false;
+        if (!(pend & kWaiting)) return;
+        pend &= ~kWaiting;
         if constexpr (F64) {
-            const i64 *b2q = reinterpret_cast<const i64 *>(sm + S::N8A) + ecol;
-            const int2 *w3q = reinterpret_cast<const int2 *>(sm + S::N8B) + ecol;
+            const i64 *b2q = reinterpret_cast<const i64 *>(sm + S::COL) + ecol;
+            const int2 *w3q = reinterpret_cast<const int2 *>(sm + S::COL + NW * 8) + ecol;
+            const int *cs = sCs + ecol, down = sc.const_x - pend_x;
             // eight columns an iteration from the front of the register array,
             // which then moves up (a run-time loop keeps the code short)
 #pragma unroll 1
             for (int c = 0; c < cpt; c += 8) {
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
-                    const i64 g = gelu_fixed(zi[k] + b2q[c + k], pend_f2, tab, a.two);
+                    const i64 g = gelu_fixed(zi[k] + shr(b2q[c + k], down), cs[c + k] - pend_x, tab, a.two);
                     // g times W3 = wh 2^27 + wl, exact: the parts' products are at most
                     // 2^57 and there are at most 32 of each
                     const int2 w = w3q[c + k];
@@ -483,19 +939,19 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
                 for (int k = 0; k + 8 < CPT; ++k) zi[k] = zi[k + 8];
             }
         } else {
-            const float2 *p2 = reinterpret_cast<const float2 *>(sm + S::N8A) + ecol;
+            const float4 *p2 = reinterpret_cast<const float4 *>(sm + S::COL) + ecol;
 #pragma unroll 1
             for (int c = 0; c < cpt; c += 8) {
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
-                    const float2 p = p2[c + k];  // b2, W3
-                    acc_f = fmaf(p.y, gelu_fast(zf[k] + p.x), acc_f);
+                    const float4 p = p2[c + k];  // b2, W3, scale of W2's row
+                    acc_f = fmaf(p.y, gelu_fast(fmaf(zf[k], p.z, p.x)), acc_f);
                 }
 #pragma unroll
                 for (int k = 0; k + 8 < CPT; ++k) zf[k] = zf[k + 8];
             }
         }
-        if (pend_last_nh) {
+        if (pend & kLastPass) {
             // sum over the four column groups of a row (group 0 is threads < 128)
             const int group = warp >> 2;
             if constexpr (F64) {
@@ -518,9 +974,9 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
                     const int lz = hi ? __clzll((i64)hi) : 64;
                     const u64 top = lz == 0 ? hi : lz == 64 ? lo : (hi << lz) | (lo >> (64 - lz));
                     const double s = (double)(neg ? -(i64)(top >> 1) : (i64)(top >> 1));
-                    // units 2^-(f2 + 53 - e3), and 2^(65 - lz) of them (2 when all is in the low word)
-                    const int e = 65 - lz - (pend_f2 + 53 - e3);
-                    emit(s * __longlong_as_double((i64)(1023 + e) << 52) + a.b3, pend_first_bg, pend_last_bg, pend_tile);
+                    // units 2^-(Q + x), and 2^(65 - lz) of them (2 when all is in the low word)
+                    const int e = 65 - lz - (sc.const_Q + pend_x);
+                    emit_pending(s * __longlong_as_double((i64)(1023 + e) << 52) + a.b3);
                 }
             } else {
                 float *pf = reinterpret_cast<float *>(sm + S::PART);
@@ -530,7 +986,7 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
                 } else {
                     wait(&part_ready, part_parity);
                     const float s = (acc_f + pf[tid]) + (pf[ROWS + tid] + pf[2 * ROWS + tid]);
-                    emit(s + (float)a.b3, pend_first_bg, pend_last_bg, pend_tile);
+                    emit_pending(s + (float)a.b3);
                 }
             }
             acc_hh = acc_hl = acc_lh = acc_ll = 0;
@@ -538,93 +994,108 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
         }
     };
 
+    auto forget = [&]() {  // what a finished pass leaves in registers
+#pragma unroll
+        for (int k = 0; k < (F64 ? CPT : 1); ++k) zi[k] = 0;
+#pragma unroll
+        for (int k = 0; k < (F64 ? 1 : CPT); ++k) zf[k] = 0.f;
+        acc_hh = acc_hl = acc_lh = acc_ll = 0;
+        acc_f = 0.f;
+    };
+
     // ---- the walk over (tile, background row, pass over layer 2, K chunk) ----
-    long long t = t_begin;
+    int t = t_begin;
     int bgi = 0, nh = 0, kc = 0;
-    long long key = -1;        // (instance, background row) the scales were made for
-    long long const_key = -1;  // key and nh of the epilogue's per-unit constants
-    int chunk_key = -1;        // last chunk (of key) that DL, dhigh and base0 were made for
-    int w_key = -1;            // (nh, kc) of the resident slices of W2 (float32: the chunks made)
-    int E = 0, f2 = 0;         // layer 1 stays below 2^E; fraction bits of layer 2 (float64)
+    int inst_now = -1, bg_now = -1;  // the instance and background row of the scales and tables in place
+    int const_nh = -1, const_version = -1;  // what the epilogue's per-unit constants were made for
+    int chunk_key = -1;        // last chunk (of them) that DL, dhigh and base0 were made for
+    int w_key = -1, w_version = -1;  // (nh, kc) of the resident slices of W2 (float32: the chunks made)
+    int rbuf = 0;              // buffer of sEr and sFlag of the tile and background row
     bool ok = false;
-    P dhigh[CHUNKS][3] = {}, base0[CHUNKS] = {};
+    i64 dhigh[CHUNKS][3] = {}, base0[CHUNKS] = {};
     // layer-1 tables: lanes 8 v + part of a warp have unit 4 warp + v of the chunk
     const int part = lane & 7, jj = 4 * warp + (lane >> 3);
 
     // The layer-1 tables of the step at (t, bgi, kc), after every warp is done
-    // with those before: scales when the instance or background row changes,
-    // then PH[e][j] = the empty coalition's pre-activation + the high features'
-    // + those of bits 3 .. 6 (pattern e).
+    // with those before: scales when the instance changes, row scales with the
+    // tile or background row, then PH[e][j] = the empty coalition's
+    // pre-activation + the high features' + those of bits 3 .. 6 (pattern e).
     auto prepare_step = [&]() {
-        const long long inst = t >> tile_shift;
-        const long long S_high = (t - (inst << tile_shift)) << LOW;
-        const double *x = a.x + inst * a.d;
+        const int inst = t >> tile_shift, S_high = (t - (inst << tile_shift)) << LOW;
+        const double *x = a.x + (long long)inst * a.d;
         const double *base = a.bg + (long long)bgi * a.d;
-        if (key != inst * a.n_bg + bgi) {
-            key = inst * a.n_bg + bgi;
+        if (inst_now != inst) {
+            // nothing of the pass before and of the tables before stays in
+            // registers over the call
+            finish_pending();
+            forget();
+#pragma unroll
+            for (int c = 0; c < CHUNKS; ++c) {
+                base0[c] = 0;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) dhigh[c][k] = 0;
+            }
+            inst_now = inst;
+            set_scales<F64>(a, x, sm, sc);
+            ok = sc.ok;
             chunk_key = -1;
-            const int j = tid >> 2, q = tid & 3;
-            float bound = 0.f, top = 0.f;
-            if (j < a.h1) {
-                for (int i = q; i < a.d; i += 4) {
-                    const float xi = (float)x[i], zi0 = (float)base[i];
-                    // (a NaN or an infinity of either carries through the second term)
-                    const float m = fmaxf(fabsf(xi), fabsf(zi0)) + 0.f * (xi + zi0);
-                    const float c = fabsf((float)a.W1[(long long)j * a.d + i]) * m;
-                    bound += c;
-                    top = fmaxf(top, c);
-                }
-                if (q == 0) bound += fabsf((float)a.b1[j]);
-            }
-            for (int o = 1; o < 4; o <<= 1) {
-                bound += __shfl_xor_sync(0xffffffffu, bound, o);
-                top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
-            }
-            const bool finite = bound < 1e20f;
-            const int e = finite ? exp_above(1.01f * bound) : 100;
-            E = block_max(e, red);
-            const bool lone = finite && e >= E - 2 && e > -100 && (bound - top) < 0.00390625f * top;
-            ok = model_ok && block_max(lone ? 1 : 0, red) == 0;
-            if constexpr (F64) {
-                ok = ok && E >= -1 && E <= 16;
-                E = max(E, 0);
-                // pre-activations of layer 2 stay below 2^ze
-                const float zb = ok ? 1.02f * pow2(E) * sL1[j] + ab2 : 0.f;
-                const int ze = block_max(exp_above(zb), red);
-                f2 = min(62, 61 - ze);
-                // (its accumulators come in units of 2^(E + ew - 55))
-                ok = ok && ze <= 18 && ze >= -5 && E + ew + f2 >= 40;
-            } else {
-                ok = ok && E > -50 && E < 60 && ew < 40;
-            }
         }
+        if (bg_now != bgi) chunk_key = -1;
+        bg_now = bgi;
+        const bool first = nh == 0 && kc == 0;
+        if (first) rbuf ^= 1;
         if (!ok) return;
+        if (first && warp >= WARPS - 4) {
+            // a row's scale: what its features and b1 can give any unit, in units of 2^E
+            const int quarter = warp - (WARPS - 4), r = 32 * quarter + lane;
+            const float m = lane < a.d ? sMW[lane] : 0.f;
+            const float mx = lane < a.d ? m * magnitude(x[lane]) : 0.f, mb = lane < a.d ? m * magnitude(base[lane]) : 0.f;
+            float sum = lane >= LOW ? (((S_high >> lane) & 1) ? mx : mb) : 0.f;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            sum += sMW[a.d];
+#pragma unroll
+            for (int k = 0; k < LOW; ++k) {
+                const float in = __shfl_sync(0xffffffffu, mx, k), out = __shfl_sync(0xffffffffu, mb, k);
+                sum += ((r >> k) & 1) ? in : out;
+            }
+            // (a row of zeros has any scale)
+            const int e = sum > 0.f ? min(0, exp_above(1.01f * sum)) : 0;
+            const unsigned flags = __ballot_sync(0xffffffffu, -e > sc.row_span) & own(quarter);
+            sEr[rbuf * ROWS + r] = max(e, -sc.row_span);
+            if (lane == 0) sFlag[rbuf][quarter] = flags;
+        }
         const int j = kc * KC + jj;
-        const bool in = j < a.h1;
+        const bool in = j < a.h1 && !(sE[j] & kDead);
         const int slot = F64 ? 0 : kc;
-        P *dl = DL + slot * (LOW * KC) + jj;
+        const int ej = (sE[j] & 255) - 64;
+        const float down = F64 ? 0.f : pow2(ej - 62);
+        i64 *dl = DL + slot * (LOW * KC) + jj;
         if (F64 ? chunk_key != kc : chunk_key < kc) {
             // every feature's contribution when it joins the coalition: the low
             // seven in shared memory, the high ones (at most three per lane) in
             // registers; and the empty coalition's sum
             chunk_key = kc;
-            const int f1 = PBITS - E;
+            const int f1 = 62 - ej;
             const double *w1 = a.W1 + (long long)(in ? j : 0) * a.d;
-            P z0 = 0, dlow = 0, dh[3];
-            if (in && part == 7) z0 = (P)fix(a.b1[j], f1);
+            i64 z0 = 0, dlow = 0, dh[3];
+            if (in && part == 7) z0 = fix(a.b1[j], f1);
             if (in && part < LOW) {
-                z0 = (P)fix(w1[part] * base[part], f1);
-                dlow = (P)fix(w1[part] * x[part], f1) - z0;
+                z0 = fix(w1[part] * base[part], f1);
+                dlow = fix(w1[part] * x[part], f1) - z0;
             }
-            if (part < LOW) dl[part * KC] = dlow;
+            if (part < LOW) {
+                dl[part * KC] = dlow;
+                if (!F64 && part < 3) DF[(slot * 3 + part) * KC + jj] = (float)dlow * down;
+            }
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 const int i = LOW + part + 8 * k;
                 dh[k] = 0;
                 if (in && i < a.d) {
-                    const P z = (P)fix(w1[i] * base[i], f1);
+                    const i64 z = fix(w1[i] * base[i], f1);
                     z0 += z;
-                    dh[k] = (P)fix(w1[i] * x[i], f1) - z;
+                    dh[k] = fix(w1[i] * x[i], f1) - z;
                 }
             }
 #pragma unroll
@@ -636,7 +1107,7 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
                 }
             __syncwarp();
         }
-        P s = slot ? base0[CHUNKS - 1] : base0[0];
+        i64 s = slot ? base0[CHUNKS - 1] : base0[0];
 #pragma unroll
         for (int k = 0; k < 3; ++k)
             if ((S_high >> (LOW + part + 8 * k)) & 1) s += slot ? dhigh[CHUNKS - 1][k] : dhigh[0][k];
@@ -646,8 +1117,13 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
 #pragma unroll
         for (int m = 0; m < 3; ++m)
             if ((part >> m) & 1) s += dl[(3 + m) * KC];
-        PH[part * KC + jj] = s;
-        PH[(part + 8) * KC + jj] = s + dl[6 * KC];
+        if constexpr (F64) {
+            PH[part * KC + jj] = s;
+            PH[(part + 8) * KC + jj] = s + dl[6 * KC];
+        } else {
+            PH[part * KC + jj] = (float)s * down;
+            PH[(part + 8) * KC + jj] = (float)(s + dl[6 * KC]) * down;
+        }
     };
     auto next_step = [&]() {  // the background row or tile after this one
         nh = kc = 0;
@@ -665,84 +1141,128 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
     }
     while (t < t_end) {
         wait(&ph_ready, ph_parity);
-        if (!ok) {
-            if (__syncthreads_or(failed ? 1 : 0)) {
-                failed = true;
-                break;
+        if (nh == 0 && kc == 0) {
+            slow = false;
+            if (!ok) {
+                // (after a barrier: see the end of the walk)
+                if (__syncthreads_or(failed ? 1 : 0)) {
+                    failed = true;
+                    break;
+                }
+                finish_pending();
+                forget();
+                const int stop = min(t_end, ((t >> tile_shift) + 1) << tile_shift);
+                slow_tiles<T>(a, t, stop, smA);
+                w_version = 0;  // W2's slices are overwritten
+                t = stop;
+                if (t < t_end) {
+                    prepare_step();
+                    arrive(&ph_ready);
+                }
+                continue;
             }
-            finish_pending();  // (after a barrier: see the end of the walk)
-            const long long inst = t >> tile_shift;
-            const T f = slow_tile<T>(a, a.x + inst * a.d, a.bg + (long long)bgi * a.d, (t - (inst << tile_shift)) << LOW, smA);
-            if (tid < ROWS) emit(f, bgi == 0, bgi == a.n_bg - 1, t);
-            next_step();
-            if (t < t_end) {
-                prepare_step();
-                arrive(&ph_ready);
+            const uint4 flags = *reinterpret_cast<const uint4 *>(sFlag[rbuf]);
+            if (flags.x | flags.y | flags.z | flags.w) {
+                if (__syncthreads_or(failed ? 1 : 0)) {
+                    failed = true;
+                    break;
+                }
+                finish_pending();
+                forget();
+                const T f = slow_rows<T>(a, t, bgi, flags, smA);
+                const unsigned quarter = warp == 0 ? flags.x : warp == 1 ? flags.y : warp == 2 ? flags.z : flags.w;
+                slow = warp < 4 && ((quarter >> lane) & 1u);
+                if (slow) emit(f, bgi == 0, bgi == a.n_bg - 1, t);
+                if (2 * slow_elems(a.h1) * (int)sizeof(T) > NS * SLICE_A) w_version = 0;
+                if (flags.x == own(0) && flags.y == own(1) && flags.z == own(2) && flags.w == own(3)) {
+                    next_step();
+                    if (t < t_end) {
+                        prepare_step();
+                        arrive(&ph_ready);
+                    }
+                    continue;
+                }
             }
-            continue;
         }
+        const int *er = sEr + rbuf * ROWS;
         // ---- layer 1: units 2u, 2u + 1 of the chunk; a warp has rows 8 warp ..
         // 8 warp + 7, split over its lanes when the chunk has at most 32 or 16
-        // units; a lane walks its rows in pairs (bit 0), the pairs in Gray-code order ----
+        // units; a lane walks its rows in pairs (bit 0) ----
         {
             const int units = min(KC, a.h1 - kc * KC);
             const int lg = units <= 16 ? 3 : units <= 32 ? 4 : 5, nb = lg - 2;
             const int u = lane & ((1 << lg) - 1), sub = lane >> lg;
-            const P *ph = PH + warp * KC + 2 * u, *dl = DL + (F64 ? 0 : kc * (LOW * KC)) + 2 * u;
+            const P *ph = PH + warp * KC + 2 * u;
             P pa = ph[0], pb = ph[1], da[3], db[3];
 #pragma unroll
             for (int m = 0; m < 3; ++m) {
-                da[m] = dl[m * KC];
-                db[m] = dl[m * KC + 1];
+                if constexpr (F64) {
+                    da[m] = DL[m * KC + 2 * u];
+                    db[m] = DL[m * KC + 2 * u + 1];
+                } else {
+                    da[m] = DF[(kc * 3 + m) * KC + 2 * u];
+                    db[m] = DF[(kc * 3 + m) * KC + 2 * u + 1];
+                }
                 if (m >= nb && ((sub >> (m - nb)) & 1)) {
                     pa += da[m];
                     pb += db[m];
                 }
             }
             const int row0 = 8 * warp + (sub << nb);
-            const float down = F64 ? 0.f : pow2(E - 30), up = F64 ? 0.f : pow2(31 - E);
+            const int2 e2 = *reinterpret_cast<const int2 *>(sE + kc * KC + 2 * u);
+            const int ea = (e2.x & 255) - 64, eb = (e2.y & 255) - 64;
+            const float ua = F64 ? 0.f : pow2(-ea), ub = F64 ? 0.f : pow2(-eb);
             auto put = [&](P za, P zb, int row) {
                 unsigned char *dst = smA + pair_offset(row, u);
                 if constexpr (F64) {
-                    // rounded to 55 fraction bits and biased
-                    const u64 c = (BIAS7 << 7) + 64;
-                    put_digits(dst, SLICE_A, ((u64)gelu_fixed(za, 62 - E, tab, a.two) + c) >> 7,
-                               ((u64)gelu_fixed(zb, 62 - E, tab, a.two) + c) >> 7);
+                    // rounded to 55 fraction bits of 2^(E + the row's exponent) and biased
+                    const int sh = 7 + er[row];
+                    const i64 c = join((lo32(BIAS7) << sh) | (1u << (sh - 1)),
+                                       (int)__funnelshift_l(lo32(BIAS7), (unsigned)hi32(BIAS7), sh));
+                    put_digits(dst, SLICE_A, (u64)shr(gelu_fixed(za, ea, tab, a.two) + c, sh),
+                               (u64)shr(gelu_fixed(zb, eb, tab, a.two) + c, sh));
                 } else {
-                    put_digits(dst, SLICE_A, (unsigned)__float2int_rn(gelu_fast((float)za * down) * up) + BIAS4,
-                               (unsigned)__float2int_rn(gelu_fast((float)zb * down) * up) + BIAS4);
+                    const float up = pow2(31 - er[row]);
+                    put_digits(dst, SLICE_A, (unsigned)__float2int_rn(gelu_fast(za) * ua * up) + BIAS4,
+                               (unsigned)__float2int_rn(gelu_fast(zb) * ub * up) + BIAS4);
                 }
             };
 #pragma unroll 1
             for (int q = 0; q < (1 << (nb - 1)); ++q) {
-                if (q == 1) {
-                    pa += da[1];
-                    pb += db[1];
-                } else if (q == 2) {
-                    pa += da[2];
-                    pb += db[2];
-                } else if (q == 3) {
-                    pa -= da[1];
-                    pb -= db[1];
+                P za = pa, zb = pb;
+                if (q & 1) {
+                    za += da[1];
+                    zb += db[1];
                 }
-                const int row = row0 + 2 * (q ^ (q >> 1));
-                put(pa, pb, row);
-                put(pa + da[0], pb + db[0], row + 1);
+                if (q & 2) {
+                    za += da[2];
+                    zb += db[2];
+                }
+                const int row = row0 + 2 * q;
+                put(za, zb, row);
+                put(za + da[0], zb + db[0], row + 1);
             }
         }
         // ---- the slices of W2 for (nh, kc) (float64: one chunk is held;
-        // float32: both, made with the first tile) ----
+        // float32: both, made with the first tile of new scales) ----
+        if (w_version != sc.version) {
+            w_version = sc.version;
+            w_key = -1;
+        }
         if (F64 ? w_key != nh * n_kc + kc : w_key < kc) {
             w_key = F64 ? nh * n_kc + kc : kc;
             unsigned char *w_dst = smW + (F64 ? 0 : kc * (NS * NW * 128));
             const int u = lane, j0 = kc * KC + 2 * u;
+            const int2 e2 = *reinterpret_cast<const int2 *>(sE + j0);
+            const int ea = BITS - 64 + (e2.x & 255), eb = BITS - 64 + (e2.y & 255);
+            const bool in_a = j0 < a.h1 && !(e2.x & kDead), in_b = j0 + 1 < a.h1 && !(e2.y & kDead);
             for (int n = warp; n < NW; n += WARPS) {
-                const int gn = nh * NW + n;
+                const int gn = nh * NW + n, ew = sEw[gn];
                 i64 wa = 0, wb = 0;
-                if (gn < a.h2) {
+                if (gn < a.h2 && ew != kDead) {
                     const double *w = a.W2 + (long long)gn * a.h1;
-                    if (j0 < a.h1) wa = fix(w[j0], BITS - ew);
-                    if (j0 + 1 < a.h1) wb = fix(w[j0 + 1], BITS - ew);
+                    if (in_a) wa = fix(w[j0], ea - ew);
+                    if (in_b) wb = fix(w[j0 + 1], eb - ew);
                 }
                 if constexpr (F64)
                     put_digits(w_dst + pair_offset(n, u), NW * 128, (u64)wa + BIAS7, (u64)wb + BIAS7);
@@ -793,8 +1313,36 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
         }
         // ---- meanwhile the tables of the next step and the pass before ----
         const bool last_kc = kc == n_kc - 1;
-        const int c_nh = nh, c_bg = bgi, c_E = E, c_f2 = f2;
-        const long long c_t = t, c_key = key;
+        const int c_nh = nh, c_bg = bgi, c_rbuf = rbuf;
+        const int c_t = t;
+        if (last_kc && (const_nh != nh || const_version != sc.version)) {
+            // per-unit constants of this pass's epilogue, while its scales are in place
+            const_nh = nh;
+            const_version = sc.version;
+            finish_pending();
+            __syncthreads();
+            if (tid == 0) {
+                sc.const_x = sc.xmax;
+                sc.const_Q = sc.Q;
+            }
+            if (tid < NW) {
+                const int gn = nh * NW + tid, ew = sEw[gn];
+                const bool in = gn < a.h2 && ew != kDead;
+                if constexpr (F64) {
+                    const int fn = sFn[gn];
+                    reinterpret_cast<i64 *>(sm + S::COL)[tid] = in ? fix(a.b2[gn], fn + sc.xmax) : 0;
+                    const i64 w = in ? fix(a.W3[gn], sc.Q - fn) : 0;  // wh 2^27 + wl, |wl| <= 2^26
+                    const int wh = (int)((w + (1ll << 26)) >> 27);
+                    reinterpret_cast<int2 *>(sm + S::COL + NW * 8)[tid] = make_int2(wh, (int)(w - ((i64)wh << 27)));
+                    sCs[tid] = 62 - fn;
+                    sCe[tid] = in ? ew + fn - 38 : 7;
+                } else {
+                    reinterpret_cast<float4 *>(sm + S::COL)[tid] =
+                        in ? make_float4((float)a.b2[gn], (float)a.W3[gn], pow2(ew), 0.f) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+            }
+            __syncthreads();
+        }
         if (!last_kc) {
             ++kc;
         } else if (nh < n_nh - 1) {
@@ -808,31 +1356,12 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
             arrive(&ph_ready);
         }
         finish_pending();
-        if (last_kc && const_key != c_key * n_nh + c_nh) {
-            // per-unit constants of this pass's epilogue
-            const_key = c_key * n_nh + c_nh;
-            __syncthreads();
-            if (tid < NW) {
-                const int gn = c_nh * NW + tid;
-                const bool in = gn < a.h2;
-                if constexpr (F64) {
-                    reinterpret_cast<i64 *>(sm + S::N8A)[tid] = in ? fix(a.b2[gn], c_f2) : 0;
-                    const i64 w = in ? fix(a.W3[gn], 53 - e3) : 0;  // wh 2^27 + wl, |wl| <= 2^26
-                    const int wh = (int)((w + (1ll << 26)) >> 27);
-                    reinterpret_cast<int2 *>(sm + S::N8B)[tid] = make_int2(wh, (int)(w - ((i64)wh << 27)));
-                } else {
-                    reinterpret_cast<float2 *>(sm + S::N8A)[tid] =
-                        in ? make_float2((float)a.b2[gn], (float)a.W3[gn]) : make_float2(0.f, 0.f);
-                }
-            }
-            __syncthreads();
-        }
         wait(&mbar, parity);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (!last_kc) continue;
         // ---- drain the accumulators of this pass into registers ----
-        const int sl = F64 ? c_E + ew + c_f2 - 38 : 0;  // from units of 2^(E + ew - 38) to the format of layer 2
-        const float zscale = F64 ? 0.f : pow2(c_E + ew - 14);
+        const int e_row = sEr[c_rbuf * ROWS + erow], x_row = min(-e_row, sc.const_x);
+        const float zscale = F64 ? 0.f : pow2(e_row - 14);
         const uint32_t lane_base = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)ecol;
         if constexpr (F64) {
 #pragma unroll
@@ -851,11 +1380,14 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
                         acc = (dg & 3) ? mad_wide(q, a.unit[dg & 3], acc) : mul_wide(q, a.unit[0]);
                     }
                 }
-                // the parts are in units of 2^(E + ew - 38) and 2^(E + ew - 70)
+                // the parts are in units of 2^(e + ew - 38) and 2^(e + ew - 70), e the row's exponent;
+                // the format of layer 2 is the unit's f and the row's x bits
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
+                for (int k = 0; k < 8; ++k) {
+                    const int sl = sCe[ecol + c + k] + e_row + x_row;
                     zi[c + k] = join(lo32(up[k]) << sl, (int)__funnelshift_l(lo32(up[k]), (unsigned)hi32(up[k]), sl)) +
                                 shr(low[k], 32 - sl);
+                }
             }
         } else {
 #pragma unroll
@@ -874,11 +1406,9 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
                 for (int k = 0; k < 8; ++k) zf[c + k] *= zscale;
             }
         }
-        pending = true;
-        pend_last_nh = c_nh == n_nh - 1;
-        pend_first_bg = c_bg == 0;
-        pend_last_bg = c_bg == a.n_bg - 1;
-        pend_f2 = c_f2;
+        pend = kWaiting | (c_nh == n_nh - 1 ? kLastPass : 0) | (c_bg == 0 ? kFirstBg : 0) |
+               (c_bg == a.n_bg - 1 ? kLastBg : 0) | (slow ? kSlow : 0);
+        pend_x = x_row;
         pend_tile = c_t;
     }
     // The row sums of the pass before may still be read by a slow warp: a pass is
@@ -887,8 +1417,9 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
     if (!failed) finish_pending();
     if (__syncthreads_or(failed ? 1 : 0)) {
         // a wait ran out (bounded): no value of this CTA's tiles is vouched for
-        for (long long i = t_begin * ROWS + tid; i < t_end * ROWS; i += THREADS)
-            reinterpret_cast<T *>(a.v)[i] = (T)__longlong_as_double(0x7ff8000000000000ll);
+        if (own_row)
+            for (int i = t_begin; i < t_end; ++i)
+                reinterpret_cast<T *>(a.v)[(long long)i * ROWS + tid] = (T)__longlong_as_double(0x7ff8000000000000ll);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -896,24 +1427,30 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
 }
 
 template <bool F64>
-static tt_fsi_status launch(const Args &a, cudaStream_t st) {
+static tt_fsi_status launch(Args a, cudaStream_t st) {
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(masked_game_split_kernel<F64>, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<F64>::BYTES);
     if (e != cudaSuccess) return TT_FSI_ERR_CUDA;
-    const unsigned grid = (unsigned)std::min<long long>(a.n_tiles, sms);
+    a.halves = 2 * a.n_tiles <= sms;
+    const unsigned grid = (unsigned)(a.halves ? 2 * a.n_tiles : std::min<long long>(a.n_tiles, sms));
     masked_game_split_kernel<F64><<<grid, THREADS, Smem<F64>::BYTES, st>>>(a);
     e = cudaGetLastError();
     if (e == cudaSuccess) return TT_FSI_OK;
     return e == cudaErrorMemoryAllocation ? TT_FSI_ERR_NO_MEMORY : TT_FSI_ERR_CUDA;
 }
 
-// Float32 models of fewer than 24 x 24 hidden units stay on masked_game_kernel:
-// a tile costs this path about 4 us of one SM whatever its width.
-bool split_serves(int d, int h1, int h2, int out_f32) {
-    return d >= LOW && h1 <= MAXH && h2 <= MAXH && (!out_f32 || h1 * h2 >= 24 * 24);
+// Narrower models stay on masked_game_kernel: a tile costs this path 7 us
+// (float64) or 4 us (float32) of one SM whatever its width (16 instances, d = 14,
+// float64: 2 x 2 units 131 us there and 116 to 182 here, by how many instances fit,
+// 4 x 4 235 and 116; float32, 24 x 24: 60.5 and 61), and in float64 the prologue of
+// a few tiles costs more than 4 x 4 units do (one instance, d = 7: 25 and 28).
+bool split_serves(int d, int h1, int h2, long long B, int out_f32) {
+    if (d < LOW || h1 > MAXH || h2 > MAXH) return false;
+    if (out_f32) return h1 * h2 >= 26 * 26;
+    return h1 + h2 >= ((B << (d - LOW)) >= 152 ? 8 : 12);
 }
 
 tt_fsi_status split_launch(const tt_fsi_mlp *model, const double *x_dev, const double *bg_dev, int n_bg, long long B,
@@ -936,6 +1473,7 @@ tt_fsi_status split_launch(const tt_fsi_mlp *model, const double *x_dev, const d
     a.h1 = model->h1;
     a.h2 = model->h2;
     a.n_tiles = B << (model->d - LOW);
+    a.halves = 0;
     a.scale = 1.0 / (double)n_bg;
     a.two = 2;
     for (int k = 0; k < 4; ++k) a.unit[k] = 1 << (24 - 8 * k);

@@ -6,7 +6,7 @@
 namespace ttfsi_mgs {
 
 // Whether the path takes a model of these sizes.
-bool split_serves(int d, int h1, int h2, int out_f32);
+bool split_serves(int d, int h1, int h2, long long B, int out_f32);
 
 // v[b, S] = mean over the n_bg rows of bg_dev of f(x_S, row elsewhere), all
 // coalitions, float64 or (out_f32) float32; arguments already checked.
