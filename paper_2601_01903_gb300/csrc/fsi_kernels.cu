@@ -1698,6 +1698,17 @@ struct BatchItem {
 template <typename Acc, int MAXL>
 constexpr int kBatchMinBlocks = MAXL > 3 || sizeof(Acc) == 8 && !TileTraits<Acc>::exact ? 2 : TileTraits<Acc>::exact ? 3 : 4;
 
+// Batches of one wave of tiles gain nothing from more CTAs per SM and lose by
+// the tile body's fewer registers and by the one thread that fetches an item's
+// arguments for all: up to three tiles per SM, exact and float32 batches run two
+// CTAs per SM whose threads each hold the arguments (ROOMY).  us per call, so
+// and with kBatchMinBlocks: float32, 30 tiles 16.8 and 18.6, 268 tiles 20.9 and
+// 23.8, 522 tiles 24.9 and 24.8; exact, 30 tiles 27.6 and 31.9, 268 tiles 33.2 and 39.5,
+// 522 tiles 39.2 and 36.2.  (float64, bound by its pipe: 30 tiles 54.9 and 51.9.)
+template <typename Acc>
+constexpr bool kBatchRoomy = TileTraits<Acc>::exact || sizeof(Acc) == 4;
+constexpr int kBatchRoomyTiles = 3;  // per SM
+
 struct BatchArgs {
     const void *v;
     void *phi;
@@ -1715,40 +1726,54 @@ struct BatchArgs {
     int inject_missing;  // test hook: every wait expects one tile more than exists
 };
 
-template <typename Acc, int MAXL>
-__global__ void __launch_bounds__(kTileThreads, kBatchMinBlocks<Acc, MAXL>) fsi_batch_kernel(BatchArgs a) {
+// The arguments of item k of a batch.
+template <typename Acc>
+__device__ __forceinline__ void batch_fetch(const BatchArgs &a, int k, BatchItem &it, FastArgs &fa, CombineFastArgs &ca) {
     using GT = typename GTraits<Acc>::G;
     using In = typename TileTraits<Acc>::In;
     using Out = typename std::conditional<sizeof(Acc) == 4, float, double>::type;
-    // the item's arguments sit in shared memory, not in every thread's registers
+    it = a.items[k];
+    const BatchGameDev g = a.games[it.game];
+    if (k < a.n_tile_items) {
+        fa = a.fplans[g.plan];
+        fa.v = reinterpret_cast<const In *>(a.v) + g.v_off;
+        fa.G = reinterpret_cast<GT *>(a.G) + g.g_off;
+        fa.tile_exp = a.tile_exp + g.exp_off;
+        fa.err = a.err;
+    } else {
+        ca = a.cplans[g.plan];
+        ca.G = reinterpret_cast<GT *>(a.G) + g.g_off;
+        ca.tile_exp = a.tile_exp + g.exp_off;
+        ca.phi = reinterpret_cast<Out *>(a.phi) + g.phi_off;
+    }
+}
+
+template <typename Acc, int MAXL, bool ROOMY>
+__global__ void __launch_bounds__(kTileThreads, ROOMY ? 2 : kBatchMinBlocks<Acc, MAXL>) fsi_batch_kernel(BatchArgs a) {
     __shared__ int s_item, s_ok;
-    __shared__ FastArgs fa;
-    __shared__ CombineFastArgs ca;
-    __shared__ BatchItem it;
+    // the item's arguments: every thread's (ROOMY), or in shared memory
+    FastArgs my_fa;
+    CombineFastArgs my_ca;
+    BatchItem my_it;
+    __shared__ FastArgs s_fa;
+    __shared__ CombineFastArgs s_ca;
+    __shared__ BatchItem s_it;
+    FastArgs &fa = ROOMY ? my_fa : s_fa;
+    CombineFastArgs &ca = ROOMY ? my_ca : s_ca;
+    BatchItem &it = ROOMY ? my_it : s_it;
     for (;;) {
         if (threadIdx.x == 0) {
             const int k = atomicAdd(a.head, 1);
             s_item = k;
-            if (k < a.n_items) {
-                it = a.items[k];
-                const BatchGameDev g = a.games[it.game];
-                if (k < a.n_tile_items) {
-                    fa = a.fplans[g.plan];
-                    fa.v = reinterpret_cast<const In *>(a.v) + g.v_off;
-                    fa.G = reinterpret_cast<GT *>(a.G) + g.g_off;
-                    fa.tile_exp = a.tile_exp + g.exp_off;
-                    fa.err = a.err;
-                } else {
-                    ca = a.cplans[g.plan];
-                    ca.G = reinterpret_cast<GT *>(a.G) + g.g_off;
-                    ca.tile_exp = a.tile_exp + g.exp_off;
-                    ca.phi = reinterpret_cast<Out *>(a.phi) + g.phi_off;
-                }
-            }
+            if (!ROOMY && k < a.n_items) batch_fetch<Acc>(a, k, it, fa, ca);
         }
         __syncthreads();
         const int item = s_item;
         if (item >= a.n_items) break;
+        if (ROOMY) {
+            __syncthreads();  // s_item is read by all before thread 0 fetches the next
+            batch_fetch<Acc>(a, item, it, fa, ca);
+        }
         if (item < a.n_tile_items) {
             for (int t = it.first; t < it.first + it.count; ++t) {
                 tile_fast_dispatch<Acc, MAXL>(fa, 0, t);
@@ -1802,6 +1827,7 @@ struct tt_fsi_batch_s {
     int *d_exp = nullptr;
     size_t smem = 0;
     int max_ell = 1;  // highest order among the fast games
+    bool roomy = false;
     int grid = 0;
     long long spin_limit = 4000000;
     int inject_missing = 0;
@@ -1843,12 +1869,20 @@ tt_fsi_status batch_build_items(tt_fsi_batch_s *b) {
     return cuda_status(e);
 }
 
-// Resident CTAs per SM of the batch kernel for these orders.
+// The batch kernel for these orders and size.
 template <typename Acc>
-cudaError_t batch_occupancy(int max_ell, size_t smem, int *occ) {
-    auto *kernel = max_ell <= 3 ? fsi_batch_kernel<Acc, 3> : fsi_batch_kernel<Acc, 4>;
+auto batch_kernel(const tt_fsi_batch_s *b) {
+    if constexpr (kBatchRoomy<Acc>)
+        if (b->roomy) return b->max_ell <= 3 ? fsi_batch_kernel<Acc, 3, true> : fsi_batch_kernel<Acc, 4, true>;
+    return b->max_ell <= 3 ? fsi_batch_kernel<Acc, 3, false> : fsi_batch_kernel<Acc, 4, false>;
+}
+
+// Its resident CTAs per SM.
+template <typename Acc>
+cudaError_t batch_occupancy(const tt_fsi_batch_s *b, int *occ) {
+    auto *kernel = batch_kernel<Acc>(b);
     cudaError_t e = allow_max_smem(kernel);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kernel, kTileThreads, smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kernel, kTileThreads, b->smem);
     return e;
 }
 
@@ -1888,10 +1922,7 @@ tt_fsi_status batch_launch(tt_fsi_batch_s *b, const void *v, void *phi, cudaStre
         a.done = b->d_counters + 1;
         a.spin_limit = b->spin_limit;
         a.inject_missing = b->inject_missing;
-        if (b->max_ell <= 3)
-            fsi_batch_kernel<Acc, 3><<<b->grid, kTileThreads, b->smem, st>>>(a);
-        else
-            fsi_batch_kernel<Acc, 4><<<b->grid, kTileThreads, b->smem, st>>>(a);
+        batch_kernel<Acc>(b)<<<std::min(b->grid, b->n_items), kTileThreads, b->smem, st>>>(a);
         e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_status(e);
     }
@@ -2005,14 +2036,13 @@ tt_fsi_status tt_fsi_batch_create_index(const tt_fsi_game *games_host, int64_t n
     if (e == cudaSuccess && eoff > 0) e = cudaMalloc((void **)&b->d_exp, (size_t)eoff * sizeof(int));
     if (e == cudaSuccess && !b->fast_games.empty()) {
         int occ = 0, dev = 0, sms = 0;
-        if (arith == TT_FSI_ARITH_EXACT)
-            e = batch_occupancy<long long>(b->max_ell, b->smem, &occ);
-        else if (arith == TT_FSI_ARITH_F64)
-            e = batch_occupancy<double>(b->max_ell, b->smem, &occ);
-        else
-            e = batch_occupancy<float>(b->max_ell, b->smem, &occ);
         if (e == cudaSuccess) e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        b->roomy = eoff <= (long long)kBatchRoomyTiles * sms;  // (an exponent per tile)
+        if (e == cudaSuccess)
+            e = arith == TT_FSI_ARITH_EXACT ? batch_occupancy<long long>(b.get(), &occ)
+                : arith == TT_FSI_ARITH_F64 ? batch_occupancy<double>(b.get(), &occ)
+                                            : batch_occupancy<float>(b.get(), &occ);
         b->grid = std::max(1, occ) * sms;  // every CTA resident at once: waits can always be served
         if (occ < 1) e = cudaErrorInvalidConfiguration;
     }
