@@ -628,6 +628,16 @@ __global__ void __launch_bounds__(kDirectThreads) fsi_direct_kernel(DirectArgs a
 // 14.4 / 12.3 at 64; d = 10, l = 2: 6.2 / 10.3, equal at 128 (2^22.8); d = 11,
 // l = 4: 8.2 / 14.4 at 4 games (2^22.1), 18.5 / 14.4 at 16.
 constexpr long long kDirectTerms = 3ll << 21;
+bool takes_direct(const Plan &p, int64_t B) {
+    return p.fast12 && !p.fused && p.d_direct && B <= 65535 && ((p.n_out * B) << p.d) <= kDirectTerms;
+}
+
+// Each of its CTAs reads the game for its eight scores, so a game in host
+// memory crosses the link n_out / 8 times.  Up to this many bytes in all that is
+// still the faster way (page-locked input, us per call, in place / copied: d = 8,
+// l = 2 22.4 / 24.5; d = 11, l = 4, 1.1 MB 31.7 / 33.3; d = 10, l = 3, 16 games, 2.8
+// MB 42.2 / 32.6); beyond it the games are copied first.
+constexpr int64_t kDirectHostBytes = 5 << 18;
 
 // ----------------------------------------------------------------------------
 // Fused apply of a fast-path plan: one persistent launch runs the tiles and
@@ -1089,7 +1099,7 @@ tt_fsi_status launch_apply(const Plan &p, const void *v, int64_t B, void *phi, c
         return TT_FSI_OK;
     }
     if constexpr (TileTraits<Acc>::exact) {
-        if (p.fast12 && p.d_direct && B <= 65535 && ((p.n_out * B) << p.d) <= kDirectTerms) {
+        if (takes_direct(p, B)) {
             DirectArgs da{};
             da.v = static_cast<const unsigned long long *>(v);
             da.phi = static_cast<double *>(phi);
@@ -1399,8 +1409,11 @@ tt_fsi_status tt_fsi_apply_host(tt_fsi_plan plan, const void *v_host, int64_t B,
     // Page-locked input: the tile kernel streams it from host memory itself.
     // It reads every input value exactly once, so the host link carries the
     // same bytes as a copy would, in one pass and without a staging buffer.
+    // (The direct kernel of small games reads them once per eight scores.)
     const void *v_mapped = nullptr;
-    if (plan->host_zero_copy) {
+    const bool few_bytes = !takes_direct(p, B) ||
+                           (int64_t)vbytes * B * ((p.n_out + kDirectWarps - 1) / kDirectWarps) <= kDirectHostBytes;
+    if (plan->host_zero_copy && few_bytes) {
         cudaPointerAttributes at{};
         if (cudaPointerGetAttributes(&at, v_host) == cudaSuccess && at.type == cudaMemoryTypeHost &&
             at.devicePointer != nullptr)
