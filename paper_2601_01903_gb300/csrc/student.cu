@@ -13,6 +13,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "gemm_tcgen05.cuh"
 #include "student_gemm.cuh"
@@ -25,21 +26,26 @@ tt_fsi_status st_status(cudaError_t e) {
     return e == cudaErrorMemoryAllocation ? TT_FSI_ERR_NO_MEMORY : TT_FSI_ERR_CUDA;
 }
 
-bool g_gemm_attr_set[64] = {false};
+std::atomic<bool> g_gemm_attr_set[64];
 
 // The driver's tensor-map encoder, looked up through the runtime (so the
 // library does not link the driver library itself); null if unavailable.
+// Safe on several threads at once: each that finds none yet looks it up.  The
+// encoder wants a current context, which a thread has only after its first
+// runtime call of some kinds: setting the device it has makes one current.
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    static bool looked = false;
-    if (!looked) {
-        looked = true;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess) return nullptr;
+    static std::atomic<PFN_cuTensorMapEncodeTiled_v12000> found{nullptr};
+    PFN_cuTensorMapEncodeTiled_v12000 fn = found.load();
+    if (!fn) {
         void *p = nullptr;
         cudaDriverEntryPointQueryResult q{};
         if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
                 cudaSuccess &&
             q == cudaDriverEntryPointSuccess)
             fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+        if (fn) found.store(fn);
     }
     return fn;
 }
