@@ -318,7 +318,9 @@ class Explainer:
         # they share one flag, read once before the residuals are returned.
         err = torch.zeros(1, dtype=torch.int32, device="cuda")
         vcoal = torch.empty((min(n, self.batch), self.K), dtype=torch.float32, device="cuda")
-        base = self.baseline.contiguous()
+        base = torch.as_tensor(self.baseline).to(device="cuda", dtype=torch.float64).contiguous()
+        if base.shape[-1] != self.d or x64.shape[-1] != self.d:
+            raise ValueError("instances and baseline rows must have d entries")
         n_bg = 1 if base.dim() == 1 else base.shape[0]
         stream = _stream_ptr()
         for s in range(0, n, self.batch):
