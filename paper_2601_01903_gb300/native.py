@@ -35,7 +35,7 @@ def sources():
 def _deps():
     files = sources()
     for name in os.listdir(_CSRC):
-        if name.endswith((".h", ".cuh")):
+        if name.endswith((".h", ".cuh", ".inc")):
             files.append(os.path.join(_CSRC, name))
     for name in os.listdir(INCLUDE):
         files.append(os.path.join(INCLUDE, name))
