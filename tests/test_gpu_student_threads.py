@@ -1,5 +1,6 @@
 """The student's first step in threads that have made no CUDA call yet (needs a
 GB300)."""
+import os
 import subprocess
 import sys
 
@@ -37,5 +38,6 @@ assert not failed, failed
 def test_first_use_from_several_threads_at_once():
     """The tensor maps are made on the first step of a student, by an encoder that
     wants a current context; it is looked up on the first step of a process."""
-    r = subprocess.run([sys.executable, "-c", _FIRST_USE], capture_output=True, text=True, timeout=200)
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _FIRST_USE], capture_output=True, text=True, timeout=200, cwd=root)
     assert r.returncode == 0, r.stderr[-2000:]
