@@ -1178,7 +1178,7 @@ tt_fsi_status launch_apply(const Plan &p, const void *v, int64_t B, void *phi, c
                     // least one batch of loads per lane (us per call at 8 lanes and
                     // now: d = 24, l = 2, one game 133.5 / 94.4; l = 1 109.1 / 69.8;
                     // d = 22, l = 3 57.2 / 47.3; d = 20, l = 3 19.0 / 16.6)
-                    const int64_t want = 2 * 152 * 32 * kC4Warps, scores = p.n_out * nb;
+                    const int64_t want = (int64_t)2 * p.sms * 32 * kC4Warps, scores = p.n_out * nb;
                     const int ql = scores * 8 >= want || p.h < 8 ? 8 : scores * 32 >= want || p.h < 11 ? 32 : 256;
                     const int per = 32 * kC4Warps / ql;
                     dim3 g2((unsigned)((p.n_out + per - 1) / per), (unsigned)nb);
@@ -1306,6 +1306,9 @@ tt_fsi_status tt_fsi_plan_create_ex(int d, int ell, tt_fsi_index index, tt_fsi_a
         }
         e = cudaMalloc((void **)&p.d_err, sizeof(int));
         if (e == cudaSuccess) e = cudaMemset(p.d_err, 0, sizeof(int));
+        int dev = 0;
+        if (e == cudaSuccess) e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p.sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) {
             st = cuda_status(e);
             break;

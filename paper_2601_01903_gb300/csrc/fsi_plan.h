@@ -72,6 +72,7 @@ struct Plan {
     // launch.  Work-item sizes and the bound on the combine's wait.
     bool fused = false;
     int tiles_per_item = 1, scores_per_item = 64;
+    int sms = 152;                          // multiprocessors of the plan's device
     int apply_grid = 0;                     // persistent CTAs (SMs x resident CTAs per SM)
     long long spin_limit = 4000000;
     bool inject_missing = false;            // test hook of the bounded wait

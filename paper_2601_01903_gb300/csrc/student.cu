@@ -468,7 +468,7 @@ int grid_for(long long n) {
 }  // namespace ttfsi_student
 
 struct tt_fsi_student_s {
-    int d = 0, H = 0, n_out = 0, n_pad = 0, max_batch = 0, ldy = 0;
+    int d = 0, H = 0, n_out = 0, n_pad = 0, max_batch = 0, ldy = 0, sms = 152;
     long long n_params = 0;
     long long off_W1 = 0, off_b1 = 0, off_W2 = 0, off_b2 = 0, off_W3 = 0, off_b3 = 0;
     float *params = nullptr, *m = nullptr, *v = nullptr, *grads = nullptr;
@@ -539,19 +539,20 @@ bool encode_map(CUtensorMap *map, CUtensorMapDataType type, int elem, const void
 // (A step of 4096 x 1024 with slices for 228 tiles, 152 and 128: 90.4, 81.3 and
 // 80.8 us; 304 cost 13 us more than 152 did: the partial sums of more slices
 // cost more than they overlap.)
-void k_split(int M, int N, int K, int &kbc, int &slices) {
+void k_split(int sms, int M, int N, int K, int &kbc, int &slices) {
     using namespace ttfsi_gemm;
     const int tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN), nk = (K + BK - 1) / BK;
-    slices = std::max(1, std::min((ttfsi_sgemm::SG_SMS + tiles - 1) / tiles, nk / 4));
+    slices = std::max(1, std::min((sms + tiles - 1) / tiles, nk / 4));
     kbc = (nk + slices - 1) / slices;
     slices = (nk + kbc - 1) / kbc;
 }
 
 int round_up(int n, int to) { return (n + to - 1) / to * to; }
 
-// A product of the step.  op = 1: the operand is stored [K, rows].
+// A product of the step, in K slices for split_sms multiprocessors (0: one slice).
+// op = 1: the operand is stored [K, rows].
 bool make_job(ttfsi_sgemm::Job &j, const bf16 *A, int lda, int a_mn, const bf16 *B, int ldb, int b_mn, int M, int N,
-              int K, bool split) {
+              int K, int split_sms) {
     using namespace ttfsi_gemm;
     const auto T = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     j.M = M;
@@ -563,7 +564,7 @@ bool make_job(ttfsi_sgemm::Job &j, const bf16 *A, int lda, int a_mn, const bf16 
     j.tiles_n = (N + BN - 1) / BN;
     int slices = 1;
     j.kbc = (K + BK - 1) / BK;
-    if (split) k_split(M, N, K, j.kbc, slices);
+    if (split_sms) k_split(split_sms, M, N, K, j.kbc, slices);
     j.zrows = round_up(M, 32);
     j.blocks = j.tiles_m * j.tiles_n * slices;
     return (a_mn ? encode_map(&j.A, T, 2, A, K, M, lda, 64, BK) : encode_map(&j.A, T, 2, A, M, K, lda, BK, BM)) &&
@@ -616,31 +617,31 @@ tt_fsi_status plan_batch(tt_fsi_student_s *s, int B) {
         j->err = s->err;
     }
     for (auto *j : {&s->f1_train, &s->f1})
-        ok = ok && make_job(j->j[0], s->Xb, d, 0, s->W1b, d, 0, B, H, d, false) &&
+        ok = ok && make_job(j->j[0], s->Xb, d, 0, s->W1b, d, 0, B, H, d, 0) &&
              out_act(j->j[0], P + s->off_b1, j == &s->f1_train ? s->Z1 : nullptr, s->A1);
     for (auto *j : {&s->f2_train, &s->f2})
-        ok = ok && make_job(j->j[0], s->A1, H, 0, s->W2b, H, 0, B, H, H, false) &&
+        ok = ok && make_job(j->j[0], s->A1, H, 0, s->W2b, H, 0, B, H, H, 0) &&
              out_act(j->j[0], P + s->off_b2, j == &s->f2_train ? s->Z2 : nullptr, s->A2);
-    ok = ok && make_job(s->f3.j[0], s->A2, H, 0, s->W3b, H, 0, B, n_out, H, true) &&
+    ok = ok && make_job(s->f3.j[0], s->A2, H, 0, s->W3b, H, 0, B, n_out, H, s->sms) &&
          out_partial(s->f3.j[0], s->Y, s->ldy);
     // dH2 = (dY W3) gelu'(Z2) and dW3 = dY^T A2
-    ok = ok && make_job(s->b3.j[0], s->dYb, n_pad, 0, s->W3b, H, 1, B, H, n_out, false) &&
+    ok = ok && make_job(s->b3.j[0], s->dYb, n_pad, 0, s->W3b, H, 1, B, H, n_out, 0) &&
          out_dgelu(s->b3.j[0], s->Z2, s->dH2, s->col2) &&
-         make_job(s->b3.j[1], s->dYb, n_pad, 1, s->A2, H, 1, n_out, H, B, true) &&
+         make_job(s->b3.j[1], s->dYb, n_pad, 1, s->A2, H, 1, n_out, H, B, s->sms) &&
          out_partial(s->b3.j[1], s->part3, H);
     // dW2 = dH2^T A1 and dH1 = (dH2 W2) gelu'(Z1)
-    ok = ok && make_job(s->b2.j[0], s->dH2, H, 1, s->A1, H, 1, H, H, B, true) &&
+    ok = ok && make_job(s->b2.j[0], s->dH2, H, 1, s->A1, H, 1, H, H, B, s->sms) &&
          out_partial(s->b2.j[0], s->part2, H) &&
-         make_job(s->b2.j[1], s->dH2, H, 0, s->W2b, H, 1, B, H, H, false) &&
+         make_job(s->b2.j[1], s->dH2, H, 0, s->W2b, H, 1, B, H, H, 0) &&
          out_dgelu(s->b2.j[1], s->Z1, s->dH1, s->col1);
     // dW1 = dH1^T X
     if (dw1_fused(s))
         ok = ok && out_dw(s->b2.j[1], s->Xb, d, s->part1);
     else
-        ok = ok && make_job(s->b1.j[0], s->dH1, H, 1, s->Xb, d, 1, H, d, B, true) && out_partial(s->b1.j[0], s->part1, d);
+        ok = ok && make_job(s->b1.j[0], s->dH1, H, 1, s->Xb, d, 1, H, d, B, s->sms) && out_partial(s->b1.j[0], s->part1, d);
     if (!ok) return TT_FSI_ERR_CUDA;
     for (auto *j : {&s->f1_train, &s->f1, &s->f2_train, &s->f2, &s->f3, &s->b3, &s->b2, &s->b1})
-        j->stages = ttfsi_sgemm::sg_stages(j->j[0].blocks + j->j[1].blocks);
+        j->stages = ttfsi_sgemm::sg_stages(j->j[0].blocks + j->j[1].blocks, s->sms);
     s->plan_B = B;
     return TT_FSI_OK;
 }
@@ -802,7 +803,9 @@ tt_fsi_status tt_fsi_student_create(int d, int hidden, int n_out, int max_batch,
     o += n_out;
     s->n_params = o;
     const size_t Bm = (size_t)max_batch, H = (size_t)hidden;
-    cudaError_t e = cudaSuccess;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, dev);
     auto A = [&](auto **p, size_t n) {
         if (e == cudaSuccess) e = st_alloc(s, p, n);
     };
@@ -832,7 +835,7 @@ tt_fsi_status tt_fsi_student_create(int d, int hidden, int n_out, int max_batch,
         // layer may have more of them at a smaller one
         int kbc, slices;
         auto rows = [&](int M, int N, int K) {
-            k_split(M, N, K, kbc, slices);
+            k_split(s->sms, M, N, K, kbc, slices);
             return (size_t)slices * round_up(M, 32);
         };
         size_t y = 0, w[3] = {0, 0, 0};

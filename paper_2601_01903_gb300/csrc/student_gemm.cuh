@@ -42,12 +42,11 @@ using namespace ttfsi_gemm;
 
 constexpr int SG_MAX_STAGES = 6;  // of 32 KB
 constexpr int SG_THREADS = 256;
-constexpr int SG_SMS = 152;
 __host__ __device__ constexpr int sg_smem(int stages) { return stages * 2 * TILE_BYTES + 1024; }
 // A CTA's loads are bound by their latency (two stages in flight: a tile of 16
 // K blocks takes 14 us alone on its SM), so a launch takes as many stages as
 // fit with the CTAs per SM that it has.
-inline int sg_stages(int blocks) { return blocks <= SG_SMS ? 6 : blocks <= 2 * SG_SMS ? 3 : 2; }
+inline int sg_stages(int blocks, int sms) { return blocks <= sms ? 6 : blocks <= 2 * sms ? 3 : 2; }
 
 enum : int { kPartial = 0, kAct = 1, kDgelu = 2 };
 
