@@ -994,13 +994,11 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
         }
     };
 
-    auto forget = [&]() {  // what a finished pass leaves in registers
+    auto forget = [&]() {  // what a finished pass leaves in registers, but for the sums of a tile's passes so far
 #pragma unroll
         for (int k = 0; k < (F64 ? CPT : 1); ++k) zi[k] = 0;
 #pragma unroll
         for (int k = 0; k < (F64 ? 1 : CPT); ++k) zf[k] = 0.f;
-        acc_hh = acc_hl = acc_lh = acc_ll = 0;
-        acc_f = 0.f;
     };
 
     // ---- the walk over (tile, background row, pass over layer 2, K chunk) ----
