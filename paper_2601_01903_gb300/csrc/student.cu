@@ -30,12 +30,8 @@ std::atomic<bool> g_gemm_attr_set[64];
 
 // The driver's tensor-map encoder, looked up through the runtime (so the
 // library does not link the driver library itself); null if unavailable.
-// Safe on several threads at once: each that finds none yet looks it up.  The
-// encoder wants a current context, which a thread has only after its first
-// runtime call of some kinds: setting the device it has makes one current.
+// Safe on several threads at once: each that finds none yet looks it up.
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess) return nullptr;
     static std::atomic<PFN_cuTensorMapEncodeTiled_v12000> found{nullptr};
     PFN_cuTensorMapEncodeTiled_v12000 fn = found.load();
     if (!fn) {
@@ -48,6 +44,13 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
         if (fn) found.store(fn);
     }
     return fn;
+}
+
+// The encoder wants a current context, which a thread has only after its first
+// runtime call of some kinds: setting the device it has makes one current.
+cudaError_t make_context_current(int &dev) {
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e == cudaSuccess ? cudaSetDevice(dev) : e;
 }
 
 // Tensor map of a row-major BF16 operand [rows, K] with row pitch ld
@@ -70,7 +73,7 @@ tt_fsi_status gemm_launch(const ttfsi_gemm::GemmArgs &a, cudaStream_t st) {
     using namespace ttfsi_gemm;
     if (a.M <= 0 || a.N <= 0 || a.K <= 0) return TT_FSI_OK;
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return TT_FSI_ERR_CUDA;
+    if (make_context_current(dev) != cudaSuccess) return TT_FSI_ERR_CUDA;
     if (dev >= 0 && dev < 64 && !g_gemm_attr_set[dev]) {
         cudaError_t e = cudaFuncSetAttribute(gemm_bf16_tcgen05, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
         if (e == cudaSuccess)
@@ -609,6 +612,8 @@ bool out_dw(ttfsi_sgemm::Job &j, const bf16 *X, int d, float *dwpart) {
 tt_fsi_status plan_batch(tt_fsi_student_s *s, int B) {
     if (s->plan_B == B) return TT_FSI_OK;
     s->plan_B = 0;
+    int dev = 0;
+    if (make_context_current(dev) != cudaSuccess) return TT_FSI_ERR_CUDA;
     const int d = s->d, H = s->H, n_out = s->n_out, n_pad = s->n_pad;
     const float *P = s->params;
     bool ok = true;
