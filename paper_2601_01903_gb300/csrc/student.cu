@@ -46,25 +46,30 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
     return fn;
 }
 
-// The encoder wants a current context, which a thread has only after its first
-// runtime call of some kinds: setting the device it has makes one current.
-cudaError_t make_context_current(int &dev) {
-    const cudaError_t e = cudaGetDevice(&dev);
-    return e == cudaSuccess ? cudaSetDevice(dev) : e;
-}
-
-// Tensor map of a row-major BF16 operand [rows, K] with row pitch ld
-// elements: 128 x 64 boxes, 128-byte swizzle, zero fill outside the matrix.
-bool operand_tensor_map(CUtensorMap *map, const __nv_bfloat16 *ptr, int rows, int K, int ld) {
+// Tensor map of a row-major array [rows, cols] with row pitch ld elements:
+// 128-byte swizzle, zero fill outside.  The encoder wants a current context,
+// which a thread has only after its first runtime call of some kinds: setting
+// the device it has makes one current.
+bool encode_map(CUtensorMap *map, CUtensorMapDataType type, int elem, const void *ptr, long long rows, int cols, int ld,
+                int box_cols, int box_rows, CUtensorMapL2promotion promotion = CU_TENSOR_MAP_L2_PROMOTION_L2_256B) {
     PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
     if (!encode) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)ld * sizeof(__nv_bfloat16)};
-    const cuuint32_t box[2] = {(cuuint32_t)ttfsi_gemm::BK, (cuuint32_t)ttfsi_gemm::BM};
+    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)ld * elem};
+    const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
-    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<__nv_bfloat16 *>(ptr), dims, strides, box,
-                  estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    auto made = [&] {
+        return encode(map, type, 2, const_cast<void *>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                      CU_TENSOR_MAP_SWIZZLE_128B, promotion, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    int dev = 0;
+    return made() || (cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess && made());
+}
+
+// A BF16 operand [rows, K] of the GEMM: boxes of 128 x 64.
+bool operand_tensor_map(CUtensorMap *map, const __nv_bfloat16 *ptr, int rows, int K, int ld) {
+    return encode_map(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ptr, rows, K, ld, ttfsi_gemm::BK, ttfsi_gemm::BM,
+                      CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
 }
 
 // Launches the TMA-fed kernel, or the cp.async kernel where an operand has
@@ -73,7 +78,7 @@ tt_fsi_status gemm_launch(const ttfsi_gemm::GemmArgs &a, cudaStream_t st) {
     using namespace ttfsi_gemm;
     if (a.M <= 0 || a.N <= 0 || a.K <= 0) return TT_FSI_OK;
     int dev = 0;
-    if (make_context_current(dev) != cudaSuccess) return TT_FSI_ERR_CUDA;
+    if (cudaGetDevice(&dev) != cudaSuccess) return TT_FSI_ERR_CUDA;
     if (dev >= 0 && dev < 64 && !g_gemm_attr_set[dev]) {
         cudaError_t e = cudaFuncSetAttribute(gemm_bf16_tcgen05, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
         if (e == cudaSuccess)
@@ -525,19 +530,6 @@ tt_fsi_status chain(void (*kernel)(P...), unsigned grid, unsigned threads, size_
     return st_status(cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...));
 }
 
-bool encode_map(CUtensorMap *map, CUtensorMapDataType type, int elem, const void *ptr, long long rows, int cols, int ld,
-                int box_cols, int box_rows) {
-    PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
-    if (!encode) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)ld * elem};
-    const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    return encode(map, type, 2, const_cast<void *>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // K slices of a product: enough for one tile per SM, at least 4 K blocks each.
 // (A step of 4096 x 1024 with slices for 228 tiles, 152 and 128: 90.4, 81.3 and
 // 80.8 us; 304 cost 13 us more than 152 did: the partial sums of more slices
@@ -612,8 +604,6 @@ bool out_dw(ttfsi_sgemm::Job &j, const bf16 *X, int d, float *dwpart) {
 tt_fsi_status plan_batch(tt_fsi_student_s *s, int B) {
     if (s->plan_B == B) return TT_FSI_OK;
     s->plan_B = 0;
-    int dev = 0;
-    if (make_context_current(dev) != cudaSuccess) return TT_FSI_ERR_CUDA;
     const int d = s->d, H = s->H, n_out = s->n_out, n_pad = s->n_pad;
     const float *P = s->params;
     bool ok = true;
