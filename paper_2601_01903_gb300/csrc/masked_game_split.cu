@@ -64,7 +64,7 @@
 //
 // Measured on one GB300: float64, 64 instances of a 14-64-64-1 model (2^20
 // coalitions) 19.67 ms on masked_game_kernel, 0.80 ms here; float32, 8
-// instances of a 16-128-128-1 model (2^19) 2.38 ms, 0.26 ms here.  Largest
+// instances of a 16-128-128-1 model (2^19) 2.38 ms, 0.27 ms here.  Largest
 // errors, coalition by coalition and against extended precision, are 0.3 to 0.9
 // of masked_game_kernel's on even models and at most 1.7 times them over units,
 // biases and features of other scales (2^-28 to 2^28, -1e8, 1e12).  An
@@ -318,10 +318,12 @@ struct Smem {
     static constexpr int SE = CE + (F64 ? C::NW * 4 : 0);       // [MAXH] exponent of a unit of layer 1 + 64, kDead
     static constexpr int EW = SE + MAXH * 4;                    // [MAXH] exponent of a row of W2, or kDead
     static constexpr int FN = EW + MAXH * 4;                    // float64: [MAXH] fraction bits of a unit of layer 2
-    static constexpr int ER = FN + (F64 ? MAXH * 4 : 0);        // [2][ROWS] exponents of the rows, double-buffered
-    static constexpr int MW = ER + 2 * ROWS * 4;                // [32] float: a feature's largest scaled weight, b1's
+    static constexpr int ER = FN + (F64 ? MAXH * 4 : 0);        // [2][ROWS], double-buffered: the rows' exponents e, a byte each | 2^(31 - e), floats
+    static constexpr int MW = ER + 2 * ROWS * (F64 ? 1 : 4);    // [32] float: a feature's largest scaled weight, b1's
     static constexpr int MB = MW + 32 * 4;                      // [32] float: a feature's largest background value
-    static constexpr int END = MB + 32 * 4;
+    static constexpr int MX = MB + 32 * 4;                      // [32] float2: what a feature gives a row, in it and not
+    static constexpr int RL = MX + 32 * 8;                      // [ROWS] float: what the low features and b1 give a row
+    static constexpr int END = RL + ROWS * 4;
     static constexpr int BYTES = END + 1024;
 };
 static_assert(Smem<true>::BYTES <= 232448 - 1024 && Smem<false>::BYTES <= 232448 - 1024, "fits one CTA per SM");
@@ -823,7 +825,9 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
     i64 *DL = reinterpret_cast<i64 *>(sm + S::DL);
     float *DF = reinterpret_cast<float *>(sm + S::DF);
     int *sE = reinterpret_cast<int *>(sm + S::SE), *sEw = reinterpret_cast<int *>(sm + S::EW);
-    int *sFn = reinterpret_cast<int *>(sm + S::FN), *sEr = reinterpret_cast<int *>(sm + S::ER);
+    int *sFn = reinterpret_cast<int *>(sm + S::FN);
+    using R = typename std::conditional<F64, signed char, float>::type;
+    R *sEr = reinterpret_cast<R *>(sm + S::ER);
     int *sCs = reinterpret_cast<int *>(sm + S::CS), *sCe = reinterpret_cast<int *>(sm + S::CE);
     const float *sMW = reinterpret_cast<const float *>(sm + S::MW);
     int *sMB = reinterpret_cast<int *>(sm + S::MB);
@@ -888,7 +892,7 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
     i64 zi[F64 ? CPT : 1];
     float zf[F64 ? 1 : CPT];
     i64 acc_hh = 0, acc_hl = 0, acc_lh = 0, acc_ll = 0;
-    float acc_f = 0.f;
+    float acc_f = 0.f, acc_f1 = 0.f;  // even and odd columns
     T vsum = 0;
     bool slow = false;  // row tid of the tile and background row came from slow_rows
     enum : int { kWaiting = 1, kLastPass = 2, kFirstBg = 4, kLastBg = 8, kSlow = 16 };
@@ -945,7 +949,8 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     const float4 p = p2[c + k];  // b2, W3, scale of W2's row
-                    acc_f = fmaf(p.y, gelu_fast(fmaf(zf[k], p.z, p.x)), acc_f);
+                    float &acc = k & 1 ? acc_f1 : acc_f;
+                    acc = fmaf(p.y, gelu_fast(fmaf(zf[k], p.z, p.x)), acc);
                 }
 #pragma unroll
                 for (int k = 0; k + 8 < CPT; ++k) zf[k] = zf[k + 8];
@@ -980,6 +985,7 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
                 }
             } else {
                 float *pf = reinterpret_cast<float *>(sm + S::PART);
+                acc_f += acc_f1;
                 if (group) {
                     pf[(group - 1) * ROWS + erow] = acc_f;
                     arrive(&part_ready);
@@ -990,15 +996,8 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
                 }
             }
             acc_hh = acc_hl = acc_lh = acc_ll = 0;
-            acc_f = 0.f;
+            acc_f = acc_f1 = 0.f;
         }
-    };
-
-    auto forget = [&]() {  // what a finished pass leaves in registers, but for the sums of a tile's passes so far
-#pragma unroll
-        for (int k = 0; k < (F64 ? CPT : 1); ++k) zi[k] = 0;
-#pragma unroll
-        for (int k = 0; k < (F64 ? 1 : CPT); ++k) zf[k] = 0.f;
     };
 
     // ---- the walk over (tile, background row, pass over layer 2, K chunk) ----
@@ -1006,13 +1005,30 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
     int bgi = 0, nh = 0, kc = 0;
     int inst_now = -1, bg_now = -1;  // the instance and background row of the scales and tables in place
     int const_nh = -1, const_version = -1;  // what the epilogue's per-unit constants were made for
-    int chunk_key = -1;        // last chunk (of them) that DL, dhigh and base0 were made for
+    // the chunk of them that DL, dhigh and base0 hold (float32: a bit for each that is held)
+    constexpr int NO_CHUNK = F64 ? -1 : 0;
+    int chunk_key = NO_CHUNK;
     int w_key = -1, w_version = -1;  // (nh, kc) of the resident slices of W2 (float32: the chunks made)
     int rbuf = 0;              // buffer of sEr and sFlag of the tile and background row
     bool ok = false;
     i64 dhigh[CHUNKS][3] = {}, base0[CHUNKS] = {};
     // layer-1 tables: lanes 8 v + part of a warp have unit 4 warp + v of the chunk
     const int part = lane & 7, jj = 4 * warp + (lane >> 3);
+    // Ahead of a call: a finished pass and the tables leave nothing in registers
+    // over it (the tables are made again) but the sums of a tile's passes so far.
+    auto forget = [&]() {
+#pragma unroll
+        for (int k = 0; k < (F64 ? CPT : 1); ++k) zi[k] = 0;
+#pragma unroll
+        for (int k = 0; k < (F64 ? 1 : CPT); ++k) zf[k] = 0.f;
+#pragma unroll
+        for (int c = 0; c < CHUNKS; ++c) {
+            base0[c] = 0;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) dhigh[c][k] = 0;
+        }
+        chunk_key = NO_CHUNK;
+    };
 
     // The layer-1 tables of the step at (t, bgi, kc), after every warp is done
     // with those before: scales when the instance changes, row scales with the
@@ -1022,45 +1038,48 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
         const int inst = t >> tile_shift, S_high = (t - (inst << tile_shift)) << LOW;
         const double *x = a.x + (long long)inst * a.d;
         const double *base = a.bg + (long long)bgi * a.d;
+        const bool new_row = inst_now != inst || bg_now != bgi;
         if (inst_now != inst) {
-            // nothing of the pass before and of the tables before stays in
-            // registers over the call
             finish_pending();
             forget();
-#pragma unroll
-            for (int c = 0; c < CHUNKS; ++c) {
-                base0[c] = 0;
-#pragma unroll
-                for (int k = 0; k < 3; ++k) dhigh[c][k] = 0;
-            }
             inst_now = inst;
             set_scales<F64>(a, x, sm, sc);
             ok = sc.ok;
-            chunk_key = -1;
         }
-        if (bg_now != bgi) chunk_key = -1;
+        if (bg_now != bgi) chunk_key = NO_CHUNK;
         bg_now = bgi;
         const bool first = nh == 0 && kc == 0;
         if (first) rbuf ^= 1;
         if (!ok) return;
         if (first && warp >= WARPS - 4) {
-            // a row's scale: what its features and b1 can give any unit, in units of 2^E
+            // a row's scale: what its features and b1 can give any unit, in units of
+            // 2^E; the low features' part once per background row (each of the four
+            // warps writes the same float2s and reads its own)
             const int quarter = warp - (WARPS - 4), r = 32 * quarter + lane;
-            const float m = lane < a.d ? sMW[lane] : 0.f;
-            const float mx = lane < a.d ? m * magnitude(x[lane]) : 0.f, mb = lane < a.d ? m * magnitude(base[lane]) : 0.f;
-            float sum = lane >= LOW ? (((S_high >> lane) & 1) ? mx : mb) : 0.f;
+            float2 *mx = reinterpret_cast<float2 *>(sm + S::MX);
+            float *low = reinterpret_cast<float *>(sm + S::RL) + r;
+            if (new_row) {
+                const float m = lane < a.d ? sMW[lane] : 0.f;
+                mx[lane] = lane < a.d ? make_float2(m * magnitude(x[lane]), m * magnitude(base[lane])) : make_float2(0.f, 0.f);
+                __syncwarp();
+                float sum = sMW[a.d];
+#pragma unroll
+                for (int k = 0; k < LOW; ++k) sum += ((r >> k) & 1) ? mx[k].x : mx[k].y;
+                *low = sum;
+            }
+            const float2 f = mx[lane];
+            float sum = lane >= LOW ? (((S_high >> lane) & 1) ? f.x : f.y) : 0.f;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            sum += sMW[a.d];
-#pragma unroll
-            for (int k = 0; k < LOW; ++k) {
-                const float in = __shfl_sync(0xffffffffu, mx, k), out = __shfl_sync(0xffffffffu, mb, k);
-                sum += ((r >> k) & 1) ? in : out;
-            }
+            sum += *low;
             // (a row of zeros has any scale)
             const int e = sum > 0.f ? min(0, exp_above(1.01f * sum)) : 0;
             const unsigned flags = __ballot_sync(0xffffffffu, -e > sc.row_span) & own(quarter);
-            sEr[rbuf * ROWS + r] = max(e, -sc.row_span);
+            const int e_row = max(e, -sc.row_span);
+            if constexpr (F64)
+                sEr[rbuf * ROWS + r] = (R)e_row;
+            else
+                sEr[rbuf * ROWS + r] = pow2(31 - e_row);
             if (lane == 0) sFlag[rbuf][quarter] = flags;
         }
         const int j = kc * KC + jj;
@@ -1069,11 +1088,11 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
         const int ej = (sE[j] & 255) - 64;
         const float down = F64 ? 0.f : pow2(ej - 62);
         i64 *dl = DL + slot * (LOW * KC) + jj;
-        if (F64 ? chunk_key != kc : chunk_key < kc) {
+        if (F64 ? chunk_key != kc : ((chunk_key >> kc) & 1) == 0) {
             // every feature's contribution when it joins the coalition: the low
             // seven in shared memory, the high ones (at most three per lane) in
             // registers; and the empty coalition's sum
-            chunk_key = kc;
+            chunk_key = F64 ? kc : chunk_key | (1 << kc);
             const int f1 = 62 - ej;
             const double *w1 = a.W1 + (long long)(in ? j : 0) * a.d;
             i64 z0 = 0, dlow = 0, dh[3];
@@ -1182,7 +1201,7 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
                 }
             }
         }
-        const int *er = sEr + rbuf * ROWS;
+        const R *er = sEr + rbuf * ROWS;
         // ---- layer 1: units 2u, 2u + 1 of the chunk; a warp has rows 8 warp ..
         // 8 warp + 7, split over its lanes when the chunk has at most 32 or 16
         // units; a lane walks its rows in pairs (bit 0) ----
@@ -1220,25 +1239,25 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
                     put_digits(dst, SLICE_A, (u64)shr(gelu_fixed(za, ea, tab, a.two) + c, sh),
                                (u64)shr(gelu_fixed(zb, eb, tab, a.two) + c, sh));
                 } else {
-                    const float up = pow2(31 - er[row]);
+                    const float up = er[row];
                     put_digits(dst, SLICE_A, (unsigned)__float2int_rn(gelu_fast(za) * ua * up) + BIAS4,
                                (unsigned)__float2int_rn(gelu_fast(zb) * ub * up) + BIAS4);
                 }
             };
 #pragma unroll 1
             for (int q = 0; q < (1 << (nb - 1)); ++q) {
-                P za = pa, zb = pb;
+                P ca = 0, cb = 0;  // (the small terms first: a float32 z has one rounding of its size)
                 if (q & 1) {
-                    za += da[1];
-                    zb += db[1];
+                    ca = da[1];
+                    cb = db[1];
                 }
                 if (q & 2) {
-                    za += da[2];
-                    zb += db[2];
+                    ca += da[2];
+                    cb += db[2];
                 }
                 const int row = row0 + 2 * q;
-                put(za, zb, row);
-                put(za + da[0], zb + db[0], row + 1);
+                put(pa + ca, pb + cb, row);
+                put(pa + (ca + da[0]), pb + (cb + db[0]), row + 1);
             }
         }
         // ---- the slices of W2 for (nh, kc) (float64: one chunk is held;
@@ -1358,8 +1377,9 @@ __global__ void __launch_bounds__(THREADS, 1) masked_game_split_kernel(const __g
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (!last_kc) continue;
         // ---- drain the accumulators of this pass into registers ----
-        const int e_row = sEr[c_rbuf * ROWS + erow], x_row = min(-e_row, sc.const_x);
-        const float zscale = F64 ? 0.f : pow2(e_row - 14);
+        const int e_row = F64 ? (int)sEr[c_rbuf * ROWS + erow] : 0, x_row = min(-e_row, sc.const_x);
+        // float32: 2^(e - 14), from the exponents of 2^(31 - e)
+        const float zscale = F64 ? 0.f : __uint_as_float((271u << 23) - __float_as_uint((float)sEr[c_rbuf * ROWS + erow]));
         const uint32_t lane_base = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)ecol;
         if constexpr (F64) {
 #pragma unroll
