@@ -337,7 +337,8 @@ tt_fsi_status tt_fsi_gemm_bf16(const void *A, int lda, const void *B, int ldb, i
  * W3 [n_out, H], b3 [n_out], concatenated.  d and H multiples of 8.
  * All *_dev arrays are FP32 device memory: x [B, d], labels [B, n_out],
  * target [B], phi [B, n_out]; loss_dev a device scalar (mean squared error
- * of the projected outputs) or NULL.  B <= max_batch.
+ * of the projected outputs) or NULL.  B <= max_batch.  The products need the
+ * driver's tensor-map encoder; without it every step is TT_FSI_ERR_CUDA.
  */
 typedef struct tt_fsi_student_s *tt_fsi_student;
 
@@ -403,7 +404,10 @@ typedef struct {
  *   v[b, S] = f(z),  z_i = x[b, i] if bit i of S is set, else baseline[i].
  *   x_dev [B, d] float64, baseline_dev [d] float64, v_dev [B, 2^d] written as
  *   float64, or float32 when out_f32 != 0 (then computed in float32, faster).
- * Asynchronous on `stream`.
+ * Asynchronous on `stream`.  A value is NaN or infinite where the model's is.
+ * The path on the tensor cores (hidden widths up to 128, d >= 7) has bounded
+ * waits inside its launch and no error word: should one run out, every value
+ * of that block's tiles (128 consecutive coalitions each) is NaN.
  */
 tt_fsi_status tt_fsi_masked_game(const tt_fsi_mlp *model, const double *x_dev,
                                  const double *baseline_dev, int64_t B, void *v_dev, int out_f32,

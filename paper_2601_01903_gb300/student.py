@@ -204,8 +204,9 @@ class Explainer:
                  baseline=None, K: int = 64, value_path: str = "tc"):
         """value_path "tc": the teacher's values for labels, spot checks and the
         fallback of ``explain`` come from the tensor-core kernel (BF16
-        layer-2 products, about 0.3 % of max|v|); "f32": from the FP32
-        CUDA-core kernels."""
+        layer-2 products, about 0.3 % of max|v|); "f32": dense values from the
+        float32 kernel (tensor cores by exact digit splitting), listed ones
+        from the FP32 CUDA-core kernel."""
         import torch
         self.torch = torch
         self.mlp = DeviceMLP(mlp, "cuda")
@@ -247,7 +248,7 @@ class Explainer:
 
     def exact(self, x64, tc=None):
         """FSI of the teacher's masked games by the exact transform (value
-        vectors in FP32 from the tensor-core or the CUDA-core kernel, widened
+        vectors in FP32 from the BF16 or the float32 kernel, widened
         to FP64)."""
         torch = self.torch
         tc = self.tc if tc is None else tc
