@@ -128,7 +128,9 @@ struct Cfg {
 // highest down: c0 (62 fraction bits), c1 (71), c2 (80; its low 16 bits hold
 // c5), c3 (57), c4 (58), c5 (59).  Largest error against 160-bit arithmetic
 // 2^-56.9, root mean square 2^-59.2 (float64's own rounding of a result near
-// 1/3 is up to 2^-55).
+// 1/3 is up to 2^-55).  The first row's c0 is 7 units lower than so rounded: the
+// integer arithmetic then gives 0 at z = 0, and a model without biases exactly b3
+// where all features are 0.
 constexpr int TAB_INTERVALS = 1120;
 constexpr int TAB_ROWS = TAB_INTERVALS + 1;
 __device__ const ulonglong2 g_gelu_table[TAB_ROWS][2] = {

@@ -166,6 +166,20 @@ def test_coalitions_of_small_values(scale):
     _check(_model(8, 48, 64, 6, 0.0), x * scale, np.zeros(8))
 
 
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("h1,h2", [(16, 20), (64, 64), (100, 128)])
+def test_features_of_zero_without_biases_give_b3(dtype, h1, h2):
+    """GELU(0) is 0 in every layer."""
+    m, x = _model(8, h1, h2, 6, 0.0), synthetic.gaussian_instances(3, 8, 15)
+    x[1, :4] = 0.0
+    x[2] = 0.0
+    for b3 in (0.0, 0.3):
+        m.b3[:] = b3
+        v = fsi.masked_game(m, x, np.zeros(8), dtype=dtype)
+        exact = torch.tensor(b3, dtype=dtype, device="cuda")
+        assert bool((v[:, 0] == exact).all() and (v[1, :16] == exact).all() and (v[2] == exact).all())
+
+
 def test_background_rows_of_different_scales():
     rows = synthetic.gaussian_instances(3, 8, 16) * np.array([[1e-3], [1.0], [50.0]])
     _check(_model(8, 64, 32, 7), synthetic.gaussian_instances(2, 8, 17), rows)
