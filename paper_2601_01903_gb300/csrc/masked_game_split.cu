@@ -698,7 +698,7 @@ __device__ __noinline__ void set_scales(const Args &a, const double *x, unsigned
         if (sc.version == 0) sc.model_e[n] = dead ? 127 : (signed char)min(e, C::EMAX);
     }
     __syncthreads();
-    // a feature's (at d: b1's) largest weight in units of 2^E
+    // the most that a feature of size 1 (at d: that b1) gives an activation, in units of 2^E
     const float unit = dead || bad ? 0.f : pow2(-e);
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
@@ -707,7 +707,8 @@ __device__ __noinline__ void set_scales(const Args &a, const double *x, unsigned
         for (int o = 4; o < 32; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
         if (lane < 4 && q + 4 * k < a.d) atomicMax(sMW + q + 4 * k, __float_as_int(m));  // none is negative
     }
-    const int b_most = __reduce_max_sync(0xffffffffu, __float_as_int(b1 * unit));
+    // (a negative bias lifts no activation; GELU is never below -0.17)
+    const int b_most = __reduce_max_sync(0xffffffffu, __float_as_int((zmax < beta ? fminf(b1, 0.18f) : b1) * unit));
     if (lane == 0) atomicMax(sMW + a.d, b_most);
 
     float wmax = 0.f, wsum = 0.f, nat = 0.f, top = 0.f;

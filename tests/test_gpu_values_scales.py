@@ -130,9 +130,9 @@ def test_half_of_the_units_of_another_scale(k):
 
 
 @pytest.mark.parametrize("b", [-20.0, -40.0, -1e3, -6e4, -1e8, 1e3])
-@pytest.mark.parametrize("layer", [1, 2])
-def test_outlying_bias(layer, b):
-    m = _model(8, 40, 48, 4)
+@pytest.mark.parametrize("layer,others", [(1, 0.1), (2, 0.1), (1, 0.0)])
+def test_outlying_bias(layer, b, others):
+    m = _model(8, 40, 48, 4, others)
     (m.b1 if layer == 1 else m.b2)[3] = b
     _check(m, synthetic.gaussian_instances(1, 8, 13), np.zeros(8))
 
